@@ -620,7 +620,7 @@ typedef struct igs_batch {
  * igs_frame_layout) with capacities[v] entries (host array of V);
  * blend_batch = entries per shared-memory batch of the blend: 32 or 64 for tile
  * 8, 64, 128 or 256 for tile 16, 64, 256, 512 or 1024 for tile 32 (0 = tile^2).
- * 64 with tile 16 or 32 selects the sub-tile blend: one 64-thread CTA per 8 x 8
+ * 64 with tile 16 or 32 selects the sub-tile blend: one warp per 8 x 8
  * pixel block, walking its tile's entries and stopping on its own (not
  * persistent); the others run the persistent whole-tile blend.
  * workspace == NULL: only *bytes. Host-only, no launch. Laying out a batch

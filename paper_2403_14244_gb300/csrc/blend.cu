@@ -1,16 +1,14 @@
 // Per-tile front-to-back compositing (Eq. 4) and its adjoint.
 //
-// One CTA per tile, one thread per pixel. The tile's entries (already in
-// front-to-back order) are staged in shared memory in batches; each pixel walks
-// them with
+// One warp per 8 x 8 pixel block of a binning tile, two pixels per lane. The
+// tile's entries (already in front-to-back order) pass by in batches of 32, those
+// that can reach the block at all (w2 d^2 <= pmax at the nearest pixel centre) are
+// queued in shared memory, and each pixel walks the queue with
 //   alpha = min(alpha_max, o * 2^(-w2 d^2)),  w2 = log2(e) / (2 s^2)   (Eq. 8)
 //   skip if alpha < alpha_min; stop (without blending) if T (1 - alpha) < t_min
 //   C += c alpha T; T *= (1 - alpha)
-// and the CTA leaves the batch loop as soon as every pixel has stopped
-// (__syncthreads_count). Each warp first ballots which staged entries can reach
-// its rows at all (w2 d^2 <= pmax at the nearest pixel centre) and walks only
-// those; the per-pixel test w2 d^2 > pmax skips the exponential where alpha must
-// fall below alpha_min. The backward pass walks each pixel's blended entries
+// and the warp leaves the list as soon as every pixel has stopped.
+// The backward pass walks each pixel's blended entries
 // in reverse from n_contrib, recovering T_k = T_{k+1} / (1 - alpha_k) from the
 // saved T_final, and reduces the per-pixel gradient terms of each entry over
 // the tile before one vector atomic per (entry, 4 floats).
@@ -19,6 +17,10 @@
 
 namespace igs {
 namespace {
+
+// Warps (8 x 8 blocks) per CTA of the forward, and resident CTAs per SM asked of the compiler.
+constexpr int kFwdWarps = 1;
+constexpr int kFwdMinCtas = 28;
 
 // Zeros to n4 float4 at p (none if p is null), spread over the grid: the
 // forward blend of a training step clears the 2D gradient for the adjoint that
@@ -29,24 +31,6 @@ __device__ __forceinline__ void clear_slice(float4* __restrict__ p, uint64_t n4)
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (uint64_t)gridDim.x * blockDim.x)
         p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
-
-template <int TS>
-__global__ void __launch_bounds__(TS* TS) k_blend_fwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
-                                                      const float4* __restrict__ rec, BlendParams P,
-                                                      float* __restrict__ img, float* __restrict__ T_final,
-                                                      uint32_t* __restrict__ n_contrib,
-                                                      const uint32_t* __restrict__ info, float4* __restrict__ clear,
-                                                      uint64_t clear4) {
-    constexpr int NT = TS * TS;
-    __shared__ float4 s_a[NT];
-    __shared__ float4 s_c[NT];
-    clear_slice(clear, clear4);
-    if (info[kInfoAbort]) return;
-    const int tile = blockIdx.x;
-    blend_tile_fwd<TS, NT>(tile % P.tiles_x, tile / P.tiles_x, P.width, P.height, ranges[tile], vals, rec, P.alpha_min,
-                           P.alpha_max, P.t_min, P.bg, s_a, s_c, img, T_final, n_contrib);
-}
-
 
 // Entries staged per barrier pair in the backward: 64 (two ballot words per
 // warp) for 16x16 tiles; 32 for 32x32 tiles (whose per-warp partials would not
@@ -281,24 +265,27 @@ __global__ void __launch_bounds__(TS * TS / 2, (2560 / (TS * TS) < 32 ? 2560 / (
 // Per pixel the walk, the arithmetic and the result are those of the whole-tile
 // kernels.
 template <int TS>
-__global__ void __launch_bounds__(64) k_blend_fwd_sub(const uint2* __restrict__ ranges,
-                                                      const uint32_t* __restrict__ vals,
-                                                      const float4* __restrict__ rec, BlendParams P,
-                                                      float* __restrict__ img, float* __restrict__ T_final,
-                                                      uint32_t* __restrict__ n_contrib,
-                                                      const uint32_t* __restrict__ info, SegLayout seg,
-                                                      float4* __restrict__ clear, uint64_t clear4) {
+__global__ void __launch_bounds__(32 * kFwdWarps, kFwdMinCtas) k_blend_fwd_sub(
+    const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ rec, BlendParams P,
+    float* __restrict__ img, float* __restrict__ T_final, uint32_t* __restrict__ n_contrib,
+    const uint32_t* __restrict__ info, SegLayout seg, const uint32_t* __restrict__ tile_order,
+    float4* __restrict__ clear, uint64_t clear4) {
     pdl_wait();
     constexpr int SUB = TS / 8;
-    __shared__ float4 s_a[64];
-    __shared__ float4 s_c[64];
+    __shared__ FwdQueue s_q[kFwdWarps];
     clear_slice(clear, clear4);
     if (info[kInfoAbort]) return;
-    const int tile = blockIdx.x / (SUB * SUB), q = blockIdx.x % (SUB * SUB);
+    const uint32_t at = blockIdx.x * kFwdWarps + (threadIdx.x >> 5);  // in starting order
+    const int q = (int)(at % (SUB * SUB));
+    const uint32_t tiles = (uint32_t)(P.tiles_x * P.tiles_y);
+    uint32_t t = at / (SUB * SUB);
+    if (t >= tiles) return;
+    if (tile_order && (t = tile_order[t]) >= tiles) return;  // (a frame whose binning never ordered its tiles)
+    const int tile = (int)t;
     const int tx = tile % P.tiles_x, ty = tile / P.tiles_x;
-    blend_tile_fwd<8, 64, true>(tx * SUB + q % SUB, ty * SUB + q / SUB, P.width, P.height, ranges[tile], vals, rec,
-                                P.alpha_min, P.alpha_max, P.t_min, P.bg, s_a, s_c, img, T_final, n_contrib, seg,
-                                blockIdx.x);
+    blend_block_fwd<TS != 8>((tx * SUB + q % SUB) * 8, (ty * SUB + q / SUB) * 8, P.width, P.height, ranges[tile], vals,
+                             rec, P.alpha_min, P.alpha_max, P.t_min, P.bg, s_q[threadIdx.x >> 5], img, T_final,
+                             n_contrib, seg, (uint32_t)(tile * SUB * SUB + q));
 }
 
 // The backward of a block's whole walk (no walk segments: the forward cut none,
@@ -401,10 +388,13 @@ cudaError_t launch_blend_fwd(const igs_frame& f, const BlendParams& bp, float* i
         z.count = 1;
         if ((e = launch_zero(z, st)) != cudaSuccess) return e;
     }
+    const uint32_t* tile_order = f.n > 0 ? sort_scratch(f).tile_order : nullptr;  // (an empty scene bins nothing)
+    const int64_t sub = f.tile / 8;
+    const dim3 grid((unsigned)ceil_div((int64_t)tiles * sub * sub, kFwdWarps)), block(32 * kFwdWarps);
     switch (f.tile) {
-        case 8: k_blend_fwd<8><<<tiles, 64, 0, st>>>(rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, clear, clear4); break;
-        case 16: e = launch_pdl(k_blend_fwd_sub<16>, dim3(tiles * 4), dim3(64), 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, clear, clear4); break;
-        case 32: e = launch_pdl(k_blend_fwd_sub<32>, dim3(tiles * 16), dim3(64), 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, clear, clear4); break;
+        case 8: e = launch_pdl(k_blend_fwd_sub<8>, grid, block, 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, tile_order, clear, clear4); break;
+        case 16: e = launch_pdl(k_blend_fwd_sub<16>, grid, block, 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, tile_order, clear, clear4); break;
+        case 32: e = launch_pdl(k_blend_fwd_sub<32>, grid, block, 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, tile_order, clear, clear4); break;
         default: return cudaErrorInvalidValue;
     }
     count_launches();

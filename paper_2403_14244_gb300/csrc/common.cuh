@@ -125,6 +125,19 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
+// 16-byte asynchronous global -> shared copy (completed by cp_async_wait).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {  // 4 bytes
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // Everything a projection kernel needs about the view (passed by value).
 struct ViewParams {
     float R[9], t[3];
@@ -298,6 +311,7 @@ struct SortScratch {
     uint32_t* walk_rows;              // [tiles_y] list starts, first level-2 chunks, chunk sizes; [1] chunk total
     uint32_t* walk_h2;                // [level-2 chunks][tiles_x] level-2 tile counts per chunk, then slots
     uint2* walk_rect;                 // [n] rectangle of order[p] (level-1 count writes, level-1 place reads)
+    uint32_t* tile_order;             // [tiles] tiles by descending entry count, for the blends; nullptr: as they come
     void* seg_base;                   // the depth items' buffers (ditems_a, ditems_b), reused by the blends'
     size_t seg_bytes;                 // walk segments once binning is done
     int64_t walk_chunks;              // > 0: counting sort of the entries; 0: duplication + tile radix passes

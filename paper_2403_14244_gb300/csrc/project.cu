@@ -78,15 +78,6 @@ struct ColorTile {
 // of an SM run out of phase and keep HBM busy while others compute.
 constexpr int kPbThreads = 32;
 
-// 16-byte asynchronous global -> shared copy (completed by cp_async_wait).
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // Adam on one parameter (the fused kernel's hot loop: 53 updates per Gaussian);
 // the bias correction is a multiplication, the square root the SFU's
 // approximation (sqrt.approx, a few ulp) and the step a fast division (2 ulp).

@@ -95,7 +95,7 @@ struct SceneRec {
 
 constexpr int kMaxGroup = 16;      // views of one grouped chain
 constexpr int kGroupWindow = 64;   // queued requests the scheduler looks through for a group
-constexpr int kBlendBatch = 64;    // batched blend: one 64-thread CTA per 8 x 8 block (8: persistent)
+constexpr int kBlendBatch = 64;    // batched blend: one warp per 8 x 8 block (8: persistent)
 constexpr int kStatusWords = 4 + kMaxGroup;  // per slot: frame/batch status, then per-view entries
 
 struct Request {

@@ -631,14 +631,47 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* 
 // exclusive offsets in place. The row's total must equal len[y], the list
 // length the row layout was built from (both count the kept Gaussians whose
 // rectangle spans row y); a difference records an error and aborts the frame
-// before any placement.
+// before any placement. With tile_order, one block more orders the tiles for the
+// blends (order_tiles) while the rows are scanned.
 constexpr int kRowScanThreads = 1024;
+
+// The tiles in descending order of their entry counts (to an eighth of a power
+// of two), for the blends: tile_order[i] is the i-th tile to start. One block, a
+// counting sort on the top bits of the count as a float. The order of equal
+// buckets is free: it decides which block starts first, not what a block computes.
+// The last blocks to start then have short lists: frames of 200K Gaussians at
+// 1001 x 667 and of 1M at 1080p take 194 and 355 us instead of 203 and 367 us.
+__device__ __forceinline__ void order_tiles(const uint2* __restrict__ ranges, uint32_t tiles,
+                                            uint32_t* __restrict__ tile_order, uint32_t* s_warp) {
+    __shared__ uint32_t s_bin[kRadix];
+    auto bin = [&](uint32_t t) {  // 0 for the largest counts
+        const uint2 r = ranges[t];
+        const uint32_t b = __float_as_uint((float)(r.y - r.x)) >> 20;  // exponent and three mantissa bits
+        return 255u - (b > 1015u ? min(b - 1015u, 255u) : 0u);         // 1016: one entry
+    };
+    for (uint32_t k = threadIdx.x; k < kRadix; k += kRowScanThreads) s_bin[k] = 0u;
+    __syncthreads();
+    for (uint32_t t = threadIdx.x; t < tiles; t += kRowScanThreads) atomicAdd(&s_bin[bin(t)], 1u);
+    __syncthreads();
+    const uint32_t c = threadIdx.x < kRadix ? s_bin[threadIdx.x] : 0u;
+    const uint32_t first = block_excl_scan<kRowScanThreads>(c, s_warp);
+    if (threadIdx.x < kRadix) s_bin[threadIdx.x] = first;
+    __syncthreads();
+    for (uint32_t t = threadIdx.x; t < tiles; t += kRowScanThreads) tile_order[atomicAdd(&s_bin[bin(t)], 1u)] = t;
+}
+
 __global__ void __launch_bounds__(kRowScanThreads) k_rows_scan(uint32_t* __restrict__ H1, uint32_t cmax,
                                                                const uint32_t* __restrict__ len,
-                                                               uint32_t* __restrict__ info) {
+                                                               uint32_t* __restrict__ info, uint32_t rows,
+                                                               const uint2* __restrict__ ranges, uint32_t tiles,
+                                                               uint32_t* __restrict__ tile_order) {
     pdl_wait();
     __shared__ uint32_t s_warp[kRowScanThreads / 32];
     if (info[kInfoAbort]) return;
+    if (blockIdx.x == rows) {  // the one block past the rows, when the tiles are to be ordered
+        order_tiles(ranges, tiles, tile_order, s_warp);
+        return;
+    }
     uint32_t* row = H1 + (size_t)blockIdx.x * cmax;
     const uint32_t used = l1_chunk(0, cmax, info).used;
     const uint32_t per = (used + kRowScanThreads - 1) / kRowScanThreads;
@@ -937,6 +970,12 @@ static int64_t l2_chunks_max(int64_t capacity, int64_t tiles_y) {
     return 2 * (ceil_div(capacity, kChunkTarget) + tiles_y) + 16;
 }
 
+// Whether a frame's tiles are ordered for the blends (order_tiles): on the counting-sort route,
+// up to as many tiles as one block orders within the level-1 scan's time. Frames of more tiles
+// have many waves of blocks, whose last one weighs little.
+constexpr int64_t kOrderTilesMax = 16384;
+static bool orders_tiles(int64_t chunks, int64_t tiles) { return chunks > 0 && tiles <= kOrderTilesMax; }
+
 // The difference grid has (tiles_y + 1)(tiles_x + 1) = tiles + tiles_x + tiles_y + 1
 // <= 2 tiles + 2 cells. Route a: vals takes 4 bytes per entry and the second
 // buffer 8 (the 8-byte level-1 items, which never outnumber the entries, live
@@ -964,6 +1003,7 @@ size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t 
     b += align256((size_t)(3 * rows + 1) * 4);                               // walk_rows
     b += align256((size_t)(chunks > 0 ? l2_chunks_max(capacity, tiles_y) * tiles_x : 0) * 4);  // walk_h2
     b += align256((size_t)(chunks > 0 ? n : 0) * 8);                         // walk_rect
+    b += align256((size_t)(orders_tiles(chunks, tiles) ? tiles : 0) * 4);    // tile_order
     return b;
 }
 
@@ -997,6 +1037,7 @@ SortScratch sort_scratch(const igs_frame& f) {
     s.walk_rows = (uint32_t*)take((size_t)(3 * rows + 1) * 4);
     s.walk_h2 = (uint32_t*)take((size_t)(chunks > 0 ? l2_chunks_max(cap, f.tiles_y) * f.tiles_x : 0) * 4);
     s.walk_rect = (uint2*)take((size_t)(chunks > 0 ? n : 0) * 8);
+    s.tile_order = orders_tiles(chunks, tiles) ? (uint32_t*)take((size_t)tiles * 4) : nullptr;
     // the last tile pass (p = passes - 1) reads items_a when p is even, items_b when odd
     const bool last_reads_a = s.tile_passes > 0 && (s.tile_passes - 1) % 2 == 0;
     s.vals = reinterpret_cast<uint32_t*>(last_reads_a ? s.items_b : s.items_a);
@@ -1120,7 +1161,8 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
         CK(launch_pdl(k_rows_count, dim3(walk_blocks((const void*)k_rows_count, count1, cmax)), dim3(32 * kWalkWarps), count1, st, f.order, rect, rows, cmax, s.walk_h1, s.walk_rect, f.info));
         count_launches();
         CK(cudaGetLastError());
-        CK(launch_pdl(k_rows_scan, dim3(rows), dim3(kRowScanThreads), 0, st, s.walk_h1, cmax, s.walk_len, f.info));
+        CK(launch_pdl(k_rows_scan, dim3(rows + (s.tile_order ? 1 : 0)), dim3(kRowScanThreads), 0, st, s.walk_h1, cmax,
+                      s.walk_len, f.info, rows, rg, (uint32_t)tiles, s.tile_order));
         count_launches();
         CK(cudaGetLastError());
         const DiscRef disc{rect, reinterpret_cast<const float4*>(f.disc), f.tile, 1.0f / (float)f.tile, footprint};
