@@ -46,3 +46,45 @@ def test_forward_walk_lengths(n, make):
     # per pixel the walk is the same whatever the binning tile
     np.testing.assert_array_equal(images[8], images[16])
     np.testing.assert_array_equal(images[8], images[32])
+
+
+def _grads(sc, W, tile):
+    r, f, scene, _ = _gpu.run_forward(sc, CAM, tile=tile)
+    g = r.run_backward(scene, CAM, f, torch.from_numpy(W.astype(np.float32)).cuda())
+    return [t.cpu().numpy().astype(np.float64) for t in g]
+
+
+@pytest.mark.parametrize("make", [_wide, _spots])
+@pytest.mark.parametrize("n", LENGTHS)
+def test_backward_walk_lengths(n, make):
+    sc = make(n)
+    W = np.random.default_rng(3).normal(size=(3, CAM.height, CAM.width)).astype(np.float32)
+    ref = oracle.backward(sc, CAM, W.astype(np.float64), mode=1)
+    for tile in (8, 16, 32):
+        d_ms, d_op, d_col = _grads(sc, W, tile)
+        _gpu.grad_close(d_ms[:, :3], ref["d_means"], f"means, tile {tile}")
+        _gpu.grad_close(d_ms[:, 3], ref["d_sigma"], f"sigma, tile {tile}")
+        _gpu.grad_close(d_op, ref["d_opac"], f"opacity, tile {tile}")
+        _gpu.grad_close(d_col, ref["d_color"].reshape(d_col.shape), f"color, tile {tile}")
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_nonfinite_image_gradient_stays_where_it_is_blended(bad):
+    # a pixel whose dL/dC is not finite reaches only the Gaussians that it blended:
+    # others of the same 8 x 8 block keep the gradients they have without it
+    sc = scene_from([[-0.30, 0.0, 0.0], [0.30, 0.0, 0.0], [0.0, 0.3, 0.0]], [0.08] * 3, [0.5] * 3, np.full((3, 3), 0.5))
+    cam = scenes.pinhole((0.0, 0.0, -2.0), 16, 16, 16.0)
+    W = np.ones((3, 16, 16), np.float32)
+    r, f, scene, _ = _gpu.run_forward(sc, cam, tile=16)
+    u, v, w2, pmax = f.rec()[:, :4].cpu().numpy().T
+    yy, xx = np.mgrid[0:16, 0:16] + 0.5
+    inside = w2[:, None, None] * ((xx - u[:, None, None]) ** 2 + (yy - v[:, None, None]) ** 2) <= pmax[:, None, None]
+    only0 = inside[0] & ~inside[1] & ~inside[2]
+    y, x = np.argwhere(only0)[0]
+    base = [t.cpu().numpy() for t in r.run_backward(scene, cam, f, torch.from_numpy(W).cuda())]
+    W[:, y, x] = bad
+    got = [t.cpu().numpy() for t in r.run_backward(scene, cam, f, torch.from_numpy(W).cuda())]
+    assert not np.isfinite(got[2][0]).all()
+    for a, b in zip(got, base):
+        # two FP32 sums of at most 256 pixels in another association: 256 x 2^-24 of the terms' size
+        np.testing.assert_allclose(a[1:], b[1:], rtol=0, atol=2e-5 * np.abs(b).max())
