@@ -6,72 +6,98 @@
 namespace igs {
 namespace {
 
-template <int DEG>
-__global__ void __launch_bounds__(256) k_project(const float4* __restrict__ ms, const float* __restrict__ op,
-                                                 const float* __restrict__ col, int64_t n, ViewParams P,
-                                                 float4* __restrict__ rec, uint2* __restrict__ rect,
-                                                 float4* __restrict__ disc, uint32_t* __restrict__ count,
-                                                 uint32_t* __restrict__ depth_key) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    project_one<DEG>(ms, op, col, i, P, rec + 2 * i, rect + i, disc + i, count + i, depth_key + i);
-}
-
-// Projection with one warp per CTA and the warp's 32 colour rows (SH degree 3)
-// staged in shared memory by coalesced 16-byte asynchronous copies (odd row
-// stride: conflict-free row reads), instead of 32 rows read lane by lane.
-constexpr int kProjRowStride = 13;  // float4 per staged row (12 used)
-
-__global__ void __launch_bounds__(32) k_project_rows3(const float4* __restrict__ ms, const float* __restrict__ op,
-                                                      const float* __restrict__ col, int64_t n, ViewParams P,
-                                                      float4* __restrict__ rec, uint2* __restrict__ rect,
-                                                      float4* __restrict__ disc, uint32_t* __restrict__ count,
-                                                      uint32_t* __restrict__ depth_key) {
-    pdl_wait();
-    __shared__ float4 s_rows[32 * kProjRowStride];
-    const int lane = threadIdx.x;
-    const int64_t wb = (int64_t)blockIdx.x * 32;
-    const int nv = (int)min((int64_t)32, n - wb);
-    const float4* src = reinterpret_cast<const float4*>(col) + wb * 12;
-    for (int q = lane; q < nv * 12; q += 32) {
-        const int g = q / 12;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                         (uint32_t)__cvta_generic_to_shared(&s_rows[g * kProjRowStride + (q - g * 12)])),
-                     "l"(src + q)
-                     : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-    if (lane >= nv) return;
-    const int64_t i = wb + lane;
-    const float4* row = s_rows + lane * kProjRowStride;
-    project_one_with<3>(ms, op, [&](float c[48]) {
-#pragma unroll
-        for (int q = 0; q < 12; ++q) {
-            const float4 v = row[q];
-            c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
-        }
-    }, i, P, rec + 2 * i, rect + i, disc + i, count + i, depth_key + i);
-}
-
-// Colour rows of a warp's 32 Gaussians are staged in shared memory (16-byte
-// asynchronous copies) so that global reads and writes of the (3 (deg+1)^2)-float
-// rows are coalesced float4 accesses; the row stride (in float4) is odd, so
-// lane-strided float4 reads of one row per lane hit distinct banks. With Adam
-// fused, the rows' moments m, v are staged the same way (dense) and stream in
-// while the warp computes the gradient.
+// Colour rows of a warp's 32 Gaussians are staged in shared memory by 16-byte
+// asynchronous copies, so that global reads and writes of the (3 (deg+1)^2)-float
+// rows are coalesced accesses: the 32 rows are one contiguous range that starts on a
+// 16-byte boundary whatever the row length. Rows of a multiple of four floats (degrees
+// 1 and 3) sit at an odd float4 stride, so lane-strided float4 reads of one row per
+// lane hit distinct banks; rows of 3 and 27 floats (RGB and degree 0, degree 2) sit
+// densely, an odd number of floats apart, for lane-strided scalar reads. (Read lane
+// by lane from global memory instead, the 27-float rows and moments of 30,000
+// Gaussians took the last pass of a training step 104 us at 0.8 % of the issue
+// slots.) With Adam fused, the rows' moments m, v are staged the same way (dense)
+// and stream in while the warp computes the gradient.
 // The gradient of coefficient (k, ch) is Y_k * drgb_ch, so instead of staging 3K
 // gradients per Gaussian the warp stages the K basis values and the 3 masked
 // colour gradients (one row of kYStride floats per Gaussian).
 template <int C>
 struct ColorTile {
-    static constexpr bool kStaged = (C % 4) == 0;
-    static constexpr int kF4 = C / 4;
-    static constexpr int kStride = kStaged ? ((kF4 % 2 == 1) ? kF4 : kF4 + 1) : 1;  // float4 units
-    static constexpr int kYStride = C / 3 + 4;                                      // K basis values + 3 (+ pad)
-    static constexpr int kWarpFloat4 = 32 * kStride + (32 * kYStride + 3) / 4;     // params, then basis rows
+    static constexpr bool kDense = (C % 4) != 0;
+    static constexpr int kF4 = C / 4;                                            // float4 per row (not dense)
+    static constexpr int kStride = kDense ? 0 : ((kF4 % 2 == 1) ? kF4 : kF4 + 1);  // float4 units
+    static constexpr int kRowsFloat4 = kDense ? 8 * C : 32 * kStride;            // the staged parameter rows
+    static constexpr int kDenseFloat4 = 8 * C;                                   // 32 rows without padding
+    static constexpr int kYStride = C / 3 + 4;                                   // K basis values + 3 (+ pad)
+    static constexpr int kWarpFloat4 = kRowsFloat4 + (32 * kYStride + 3) / 4;    // params, then basis rows
+    // this lane's row in the staged tile, as floats
+    __device__ static __forceinline__ const float* row(const float4* tile, int lane) {
+        return reinterpret_cast<const float*>(tile) + lane * (kDense ? C : 4 * kStride);
+    }
+    // float4 q of the 32 dense rows -> its place in the staged tile
+    __device__ static __forceinline__ int at(int q) {
+        if constexpr (kDense) return q;
+        const int g = q / kF4;
+        return g * kStride + (q - g * kF4);
+    }
 };
+
+// Copy the nv * C floats at src (16-byte aligned) into dst, dense.
+template <int C>
+__device__ __forceinline__ void stage_dense(float4* dst, const float* __restrict__ src, int nv, int lane) {
+    const int n4 = nv * C / 4;
+    for (int q = lane; q < n4; q += 32) cp_async16(&dst[q], reinterpret_cast<const float4*>(src) + q);
+    const int e = 4 * n4 + lane;  // the last 0..3 floats (a partial warp's)
+    if (C % 4 != 0 && e < nv * C) cp_async4(reinterpret_cast<float*>(dst) + e, src + e);
+}
+// Copy the colour rows of nv Gaussians from src into the staged tile.
+template <int C>
+__device__ __forceinline__ void stage_rows(float4* tile, const float* __restrict__ src, int nv, int lane) {
+    if constexpr (ColorTile<C>::kDense) {
+        stage_dense<C>(tile, src, nv, lane);
+    } else {
+        for (int q = lane; q < nv * ColorTile<C>::kF4; q += 32)
+            cp_async16(&tile[ColorTile<C>::at(q)], reinterpret_cast<const float4*>(src) + q);
+    }
+}
+// This lane's staged row into c[0 .. C).
+template <int C>
+__device__ __forceinline__ void read_row(const float4* tile, int lane, float c[48]) {
+    if constexpr (ColorTile<C>::kDense) {
+        const float* row = ColorTile<C>::row(tile, lane);
+#pragma unroll
+        for (int k = 0; k < C; ++k) c[k] = row[k];
+    } else {
+        const float4* row = tile + lane * ColorTile<C>::kStride;
+#pragma unroll
+        for (int q = 0; q < C / 4; ++q) {
+            const float4 v = row[q];
+            c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
+        }
+    }
+}
+
+// Projection with one warp per CTA and the warp's 32 colour rows staged in shared memory.
+template <int DEG>
+__global__ void __launch_bounds__(32) k_project_rows(const float4* __restrict__ ms, const float* __restrict__ op,
+                                                     const float* __restrict__ col, int64_t n, ViewParams P,
+                                                     float4* __restrict__ rec, uint2* __restrict__ rect,
+                                                     float4* __restrict__ disc, uint32_t* __restrict__ count,
+                                                     uint32_t* __restrict__ depth_key) {
+    pdl_wait();
+    constexpr int C = DEG < 0 ? 3 : 3 * (DEG + 1) * (DEG + 1);
+    __shared__ float4 s_rows[ColorTile<C>::kRowsFloat4];
+    const int lane = threadIdx.x;
+    const int64_t wb = (int64_t)blockIdx.x * 32;
+    const int nv = (int)min((int64_t)32, n - wb);
+    stage_rows<C>(s_rows, col + (size_t)C * (size_t)wb, nv, lane);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    if (lane >= nv) return;
+    const int64_t i = wb + lane;
+    project_one_with<DEG>(ms, op, [&](float c[48]) { read_row<C>(s_rows, lane, c); }, i, P, rec + 2 * i, rect + i,
+                          disc + i, count + i, depth_key + i);
+}
 
 // One warp per CTA: a CTA's shared memory (21.5 KB with the Adam moments staged)
 // is released as soon as its 32 Gaussians are done, so the ten resident warps
@@ -137,38 +163,28 @@ __global__ void __launch_bounds__(kPbThreads, 10) k_project_bwd(float4* __restri
     const int nv = (int)min((int64_t)32, n - wb);
     const int64_t i = wb + lane;
     const bool active = lane < nv;
-    constexpr int kWarpF4 = CT::kWarpFloat4 + (ADAM && CT::kStaged ? 2 * 32 * CT::kF4 : 0);
-    float4* A = s_tiles + (size_t)w * kWarpF4;                   // this warp's parameter rows
-    float* Ys = reinterpret_cast<float*>(A + 32 * CT::kStride);  // this warp's basis rows
-    float* Af = reinterpret_cast<float*>(A) + lane * CT::kStride * 4;
-    float4* Mrows = A + CT::kWarpFloat4;                         // Adam moments of the colour rows (dense)
-    float4* Vrows = Mrows + 32 * CT::kF4;
-    if constexpr (CT::kStaged) {
-        const float4* src = reinterpret_cast<const float4*>(col) + wb * CT::kF4;
-        for (int q = lane; q < nv * CT::kF4; q += 32) {
-            const int g = q / CT::kF4;
-            cp_async16(&A[g * CT::kStride + (q - g * CT::kF4)], src + q);
-        }
+    constexpr int kWarpF4 = CT::kWarpFloat4 + (ADAM ? 2 * CT::kDenseFloat4 : 0);
+    float4* A = s_tiles + (size_t)w * kWarpF4;                    // this warp's parameter rows
+    float* Ys = reinterpret_cast<float*>(A + CT::kRowsFloat4);    // this warp's basis rows
+    const float* Af = CT::row(A, lane);
+    float4* Mrows = A + CT::kWarpFloat4;                          // Adam moments of the colour rows (dense)
+    float4* Vrows = Mrows + CT::kDenseFloat4;
+    const size_t row0 = (size_t)C * (size_t)wb;  // the warp's first colour float
+    stage_rows<C>(A, col + row0, nv, lane);
+    cp_async_commit();
+    if constexpr (ADAM) {  // the colour moments stream in while the gradient is computed
+        stage_dense<C>(Mrows, st.m_col + row0, nv, lane);
+        stage_dense<C>(Vrows, st.v_col + row0, nv, lane);
         cp_async_commit();
-        if constexpr (ADAM) {  // the colour moments stream in while the gradient is computed
-            const float4* m4 = reinterpret_cast<const float4*>(st.m_col) + wb * CT::kF4;
-            const float4* v4 = reinterpret_cast<const float4*>(st.v_col) + wb * CT::kF4;
-            for (int q = lane; q < nv * CT::kF4; q += 32) {
-                cp_async16(&Mrows[q], m4 + q);
-                cp_async16(&Vrows[q], v4 + q);
-            }
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncwarp();
+        cp_async_wait<1>();
+    } else {
+        cp_async_wait<0>();
     }
+    __syncwarp();
     float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
     float raw_op = 0.f;
     float dmx = 0.f, dmy = 0.f, dmz = 0.f, dsig_out = 0.f, dop_out = 0.f;
-    // colour coefficients of this lane's Gaussian (staged rows, or its own strided row)
-    auto coef = [&](int k) -> float { return CT::kStaged ? Af[k] : col[(size_t)C * (size_t)i + k]; };
+    auto coef = [&](int k) -> float { return Af[k]; };  // colour coefficients of this lane's Gaussian
     bool has_grad = false;
     float drgb[3] = {0.f, 0.f, 0.f}, draw[3] = {0.f, 0.f, 0.f};
     float Y[16];
@@ -211,6 +227,10 @@ __global__ void __launch_bounds__(kPbThreads, 10) k_project_bwd(float4* __restri
         dsig_out = P.param_mode == 1 ? dsg * sg : dsg;
         dop_out = P.param_mode == 1 ? ga.w * o * (1.f - o) : ga.w;
         drgb[0] = gb.x; drgb[1] = gb.y; drgb[2] = gb.z;
+        if constexpr (DEG < 0) {  // plain colour: one basis value of 1
+            Y[0] = 1.f;
+            draw[0] = drgb[0]; draw[1] = drgb[1]; draw[2] = drgb[2];
+        }
         if constexpr (DEG >= 0) {
             dx = m.x - P.cam_center[0]; dy = m.y - P.cam_center[1]; dz = m.z - P.cam_center[2];
             const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
@@ -240,11 +260,6 @@ __global__ void __launch_bounds__(kPbThreads, 10) k_project_bwd(float4* __restri
             dmz += (gd2 - dot * dz) * inv;
         }
     }
-    // gradient of colour coefficient k (zero for culled Gaussians)
-    auto dcoef = [&](int k) -> float {
-        if constexpr (DEG < 0) return drgb[k];
-        else return Y[k / 3] * draw[k % 3];
-    };
     // means, sigma, opacity: one lane per Gaussian (coalesced rows of 16 and 4 bytes)
     ProjGeom pg{};
     if (active) {
@@ -265,17 +280,22 @@ __global__ void __launch_bounds__(kPbThreads, 10) k_project_bwd(float4* __restri
         }
     }
     // colour rows
-    if constexpr (CT::kStaged) {
-        constexpr int K = C / 3;
-        if (active) {
-            float* yr = Ys + lane * CT::kYStride;
+    constexpr int K = C / 3;
+    if (active) {
+        float* yr = Ys + lane * CT::kYStride;
 #pragma unroll
-            for (int k = 0; k < K; ++k) yr[k] = has_grad ? Y[k] : 0.f;
-            yr[K] = draw[0]; yr[K + 1] = draw[1]; yr[K + 2] = draw[2];
-        }
-        if constexpr (ADAM) cp_async_wait<0>();
-        __syncwarp();
-        const size_t row0 = (size_t)wb * CT::kF4;
+        for (int k = 0; k < K; ++k) yr[k] = has_grad ? Y[k] : 0.f;
+        yr[K] = draw[0]; yr[K + 1] = draw[1]; yr[K + 2] = draw[2];
+    }
+    if constexpr (ADAM) cp_async_wait<0>();
+    __syncwarp();
+    // gradient of the warp's colour float e (zero for culled Gaussians)
+    auto grad_at = [&](int e) -> float {
+        const int g = e / C, c = e - g * C;
+        const float* yr = Ys + g * CT::kYStride;
+        return yr[c / 3] * yr[K + c % 3];
+    };
+    if constexpr (!CT::kDense) {
 #pragma unroll 6
         for (int q = lane; q < nv * CT::kF4; q += 32) {
             const int g = q / CT::kF4;
@@ -292,43 +312,41 @@ __global__ void __launch_bounds__(kPbThreads, 10) k_project_bwd(float4* __restri
                 float4 vv = Vrows[q];
                 adam_update4(p4, g4, mm, vv, a);
                 if constexpr (NEXT) A[g * CT::kStride + (q - g * CT::kF4)] = p4;  // for the next view's colour
-                reinterpret_cast<float4*>(col)[row0 + q] = p4;
-                reinterpret_cast<float4*>(st.m_col)[row0 + q] = mm;
-                reinterpret_cast<float4*>(st.v_col)[row0 + q] = vv;
+                reinterpret_cast<float4*>(col + row0)[q] = p4;
+                reinterpret_cast<float4*>(st.m_col + row0)[q] = mm;
+                reinterpret_cast<float4*>(st.v_col + row0)[q] = vv;
             } else {
-                reinterpret_cast<float4*>(d_col)[row0 + q] = g4;
+                reinterpret_cast<float4*>(d_col + row0)[q] = g4;
             }
         }
-    } else if (active) {
-        const size_t r = (size_t)C * (size_t)i;
-#pragma unroll
-        for (int k = 0; k < C; ++k) {
-            const float gk = has_grad ? dcoef(k) : 0.f;
-            if constexpr (ADAM) {
-                float pk = col[r + k], mk = st.m_col[r + k], vk = st.v_col[r + k];
-                adam_update(pk, gk, mk, vk, a);
-                col[r + k] = pk; st.m_col[r + k] = mk; st.v_col[r + k] = vk;
-            } else {
-                d_col[r + k] = gk;
-            }
+    } else if constexpr (ADAM) {
+        const int n4 = nv * C / 4;
+        for (int q = lane; q < n4; q += 32) {  // four floats of the dense rows, which may end one row and start the next
+            const float4 g4 = make_float4(grad_at(4 * q), grad_at(4 * q + 1), grad_at(4 * q + 2), grad_at(4 * q + 3));
+            float4 p4 = A[q], mm = Mrows[q], vv = Vrows[q];
+            adam_update4(p4, g4, mm, vv, a);
+            if constexpr (NEXT) A[q] = p4;
+            reinterpret_cast<float4*>(col + row0)[q] = p4;
+            reinterpret_cast<float4*>(st.m_col + row0)[q] = mm;
+            reinterpret_cast<float4*>(st.v_col + row0)[q] = vv;
         }
+        const int e = 4 * n4 + lane;  // the last 0..3 floats (a partial warp's)
+        if (e < nv * C) {
+            float pk = reinterpret_cast<float*>(A)[e], mk = reinterpret_cast<float*>(Mrows)[e],
+                  vk = reinterpret_cast<float*>(Vrows)[e];
+            adam_update(pk, grad_at(e), mk, vk, a);
+            if constexpr (NEXT) reinterpret_cast<float*>(A)[e] = pk;
+            col[row0 + e] = pk; st.m_col[row0 + e] = mk; st.v_col[row0 + e] = vk;
+        }
+    } else {  // (d_col of such rows need not be 16-byte aligned)
+        for (int e = lane; e < nv * C; e += 32) d_col[row0 + e] = grad_at(e);
     }
     if constexpr (NEXT) {  // the next view's colour from the updated coefficients
         static_assert(ADAM, "the next view is projected from the updated parameters");
-        if constexpr (CT::kStaged) __syncwarp();  // the staged rows hold the updated coefficients
+        __syncwarp();  // the staged rows hold the updated coefficients
         if (active && pg.keep) {
             float c[48];
-            if constexpr (CT::kStaged) {
-                const float4* row = A + lane * CT::kStride;  // odd float4 stride: conflict-free
-#pragma unroll
-                for (int q = 0; q < CT::kF4; ++q) {
-                    const float4 t = row[q];
-                    c[4 * q] = t.x; c[4 * q + 1] = t.y; c[4 * q + 2] = t.z; c[4 * q + 3] = t.w;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < C; ++k) c[k] = col[(size_t)C * (size_t)i + k];  // this thread's own writes
-            }
+            read_row<C>(A, lane, c);
             project_color<DEG>(m, pg, c, P2, o2.rec + 2 * i);
         }
     }
@@ -340,8 +358,7 @@ cudaError_t launch_pb(const igs_scene& sc, const ViewParams& vp, const igs_frame
                       const ViewParams& vp2 = ViewParams{}, const ProjOut& o2 = ProjOut{}) {
     constexpr int C = DEG < 0 ? 3 : 3 * (DEG + 1) * (DEG + 1);
     const size_t smem = (size_t)(kPbThreads / 32) *
-                        (ColorTile<C>::kWarpFloat4 + (ADAM && ColorTile<C>::kStaged ? 2 * 32 * ColorTile<C>::kF4 : 0)) *
-                        sizeof(float4);
+                        (ColorTile<C>::kWarpFloat4 + (ADAM ? 2 * ColorTile<C>::kDenseFloat4 : 0)) * sizeof(float4);
     auto k = k_project_bwd<DEG, ADAM, NEXT>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -392,30 +409,23 @@ cudaError_t launch_adam_advance(int32_t* state, double lr, double b1, double b2,
 
 cudaError_t launch_project(const igs_scene& sc, const ViewParams& vp, const igs_frame& f, cudaStream_t st) {
     if (sc.n == 0) return cudaSuccess;
-    const int threads = 256;
-    const unsigned blocks = (unsigned)ceil_div(sc.n, threads);
     auto ms = reinterpret_cast<const float4*>(sc.means_sigma);
-    auto rec = reinterpret_cast<float4*>(f.rec);
-    auto rect = reinterpret_cast<uint2*>(f.rect);
-#define IGS_PROJ(D) k_project<D><<<blocks, threads, 0, st>>>(ms, sc.opacity, sc.color, sc.n, vp, rec, rect, reinterpret_cast<float4*>(f.disc), f.count, f.depth_key)
-    if (vp.sh_degree == 3 && (reinterpret_cast<uintptr_t>(sc.color) & 15) == 0) {
-        cudaError_t e = launch_pdl(k_project_rows3, dim3((unsigned)ceil_div(sc.n, 32)), dim3(32), 0, st, ms,
-                                   sc.opacity, sc.color, sc.n, vp, rec, rect, reinterpret_cast<float4*>(f.disc),
-                                   f.count, f.depth_key);
-        count_launches();
-        return e != cudaSuccess ? e : cudaGetLastError();
-    }
+    auto launch = [&](auto kernel) {  // (colour rows are 16-byte aligned: igs_project checks)
+        return launch_pdl(kernel, dim3((unsigned)ceil_div(sc.n, 32)), dim3(32), 0, st, ms, sc.opacity, sc.color, sc.n,
+                          vp, reinterpret_cast<float4*>(f.rec), reinterpret_cast<uint2*>(f.rect),
+                          reinterpret_cast<float4*>(f.disc), f.count, f.depth_key);
+    };
+    cudaError_t e;
     switch (vp.sh_degree) {
-        case -1: IGS_PROJ(-1); break;
-        case 0: IGS_PROJ(0); break;
-        case 1: IGS_PROJ(1); break;
-        case 2: IGS_PROJ(2); break;
-        case 3: IGS_PROJ(3); break;
+        case -1: e = launch(k_project_rows<-1>); break;
+        case 0: e = launch(k_project_rows<0>); break;
+        case 1: e = launch(k_project_rows<1>); break;
+        case 2: e = launch(k_project_rows<2>); break;
+        case 3: e = launch(k_project_rows<3>); break;
         default: return cudaErrorInvalidValue;
     }
-#undef IGS_PROJ
     count_launches();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_project_bwd(const igs_scene& sc, const ViewParams& vp, const igs_frame& f, const float* g2d,
