@@ -138,6 +138,16 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// b^t by squaring, t >= 0: at most 2 log2(t) FP64 products in a row (pow() runs several
+// hundred FP64 instructions, which this part issues slowly), each rounded once, so the
+// result is within 4 log2(t) 2^-53 of b^t.
+__device__ __forceinline__ double pow_int(double b, int t) {
+    double p = 1.0;
+    for (; t > 0; t >>= 1, b *= b)
+        if (t & 1) p *= b;
+    return p;
+}
+
 // Everything a projection kernel needs about the view (passed by value).
 struct ViewParams {
     float R[9], t[3];

@@ -185,11 +185,14 @@ __global__ void __launch_bounds__(256) k_fit2d_adam(float4* __restrict__ p, cons
                                                    Fit2dAdam a, int32_t* __restrict__ state) {
     __shared__ float s_step[8];
     __shared__ float s_bc2_sqrt;
-    if (threadIdx.x == 0) {
+    // (thread j < 8 forms slot j's step, thread 32 the second moment's correction: FP64 latencies side
+    // by side, 15 us for 1000 particles with pow() and eight divisions one after another on one thread)
+    if (threadIdx.x < 8 || threadIdx.x == 32) {
         const int t = state[0] + 1;
-        const double bc1 = 1.0 - pow(a.b1d, (double)t), bc2 = 1.0 - pow(a.b2d, (double)t);
-        for (int j = 0; j < 8; ++j) s_step[j] = (float)((double)a.lr[j] / bc1);
-        s_bc2_sqrt = (float)sqrt(bc2);
+        if (threadIdx.x == 32)
+            s_bc2_sqrt = (float)sqrt(1.0 - pow_int(a.b2d, t));
+        else
+            s_step[threadIdx.x] = (float)((double)a.lr[threadIdx.x] / (1.0 - pow_int(a.b1d, t)));
     }
     __syncthreads();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {

@@ -388,21 +388,27 @@ cudaError_t dispatch_pb(const igs_scene& sc, const ViewParams& vp, const igs_fra
     }
 }
 
+// One warp; lanes 0 and 1 form the two bias corrections side by side (a chain of FP64
+// latencies: 9 us with pow() on one thread, which a training step waits for).
 __global__ void k_adam_advance(int32_t* __restrict__ state, double lr, double b1, double b2) {
     pdl_wait();
     const int t = state[0] + 1;
-    state[0] = t;
-    const double bc1 = 1.0 - pow(b1, (double)t), bc2 = 1.0 - pow(b2, (double)t);
+    __syncwarp();
     float* f = reinterpret_cast<float*>(state + 1);
-    f[0] = (float)(lr / bc1);
-    f[1] = (float)(1.0 / sqrt(bc2));
-    f[2] = (float)sqrt(bc2);
+    if (threadIdx.x == 0) {
+        state[0] = t;
+        f[0] = (float)(lr / (1.0 - pow_int(b1, t)));
+    } else if (threadIdx.x == 1) {
+        const double s = sqrt(1.0 - pow_int(b2, t));
+        f[1] = (float)(1.0 / s);
+        f[2] = (float)s;
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_adam_advance(int32_t* state, double lr, double b1, double b2, cudaStream_t st) {
-    cudaError_t e = launch_pdl(k_adam_advance, dim3(1), dim3(1), 0, st, state, lr, b1, b2);
+    cudaError_t e = launch_pdl(k_adam_advance, dim3(1), dim3(32), 0, st, state, lr, b1, b2);
     count_launches();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
