@@ -329,6 +329,16 @@ struct SortScratch {
     int tile_bits;
 };
 SortScratch sort_scratch(const igs_frame& f);
+// The binning of few Gaussians in two or three launches (binsmall.cu): whether a frame takes it, and
+// its launches. The line lies where the two routes meet: 16384 Gaussians take 21-23 us against 82-96 (16-
+// and 32-pixel tiles, 320 x 240 to 1920 x 1080 pixels), 32768 30-33 against 86-97, 65536 54-58
+// against 89-102, 98304 89-95 against 92-102; with 8-pixel tiles at 1297 x 840, 32768 88 against 149,
+// 65536 150 against 168, 98304 224 against 186. (The pieces of the small route grow with n^2 / 1024 and
+// n times the strips.) More tile rows than kBinSmallRows would not fit the merge's row counters.
+constexpr int64_t kBinSmallMax = 65536;
+constexpr int64_t kBinSmallRows = 512;
+bool bin_small_ok(const igs_frame& f, int footprint);
+cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStream_t st);
 size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t tiles_y, int64_t chunks);
 
 // Walk segments of the one-view blends (16- and 32-pixel binning tiles, one

@@ -1062,6 +1062,8 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
     const int gx = f.tiles_x + 1, gy = f.tiles_y + 1;
     cudaError_t e;
 #define CK(x) do { if ((e = (x)) != cudaSuccess) { g_failed_call = #x " (sort.cu:" IGS_STR(__LINE__) ")"; return e; } } while (0)
+    // few Gaussians: a route of its own (the look-back test needs a sort with a look-back)
+    if (bin_small_ok(f, footprint) && !g_silence_next.load()) return launch_bin_small(f, s, st);
     // reset state: status words, histograms, counters, look-back words, difference grid (one launch)
     {
         ZeroRanges z = {};
