@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(TS* TS) k_blend_persistent(const BatchView* __
         const uint32_t t = w - bv.tile_base;
         blend_tile_fwd<TS, B>((int)(t % (uint32_t)vp.tiles_x), (int)(t / (uint32_t)vp.tiles_x), vp.width, vp.height,
                               bv.ranges[t], bv.vals, bv.rec, P.alpha_min, P.alpha_max, P.t_min, P.bg, s_a, s_c,
-                              images + bv.img_off, nullptr, nullptr);
+                              images + bv.img_off);
     }
 }
 

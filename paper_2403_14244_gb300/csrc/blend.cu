@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_sub(
 // The backward over walk segments: one-warp CTAs, all resident, take work from
 // one counter: first the segments the forward closed, then each block's last
 // segment (its whole walk when it closed none). Every piece walks at most
-// kSegStride list positions (unless the pool ran out), so no block's long walk
+// seg.stride list positions (unless the pool ran out), so no block's long walk
 // sets the kernel's length.
 template <int TS>
 __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_segs(const uint2* __restrict__ ranges,
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_segs(const uint2*
         const int tile = (int)(block / (SUB * SUB)), q = (int)(block % (SUB * SUB));
         const int tx = tile % P.tiles_x, ty = tile / P.tiles_x;
         blend_block_bwd((tx * SUB + q % SUB) * 8, (ty * SUB + q / SUB) * 8, ranges[tile], vals, rec, P, dL, T_final,
-                        n_contrib, g2d, s_q, lo, hi, slot == kSegNone ? nullptr : seg.pool + (size_t)slot * 64);
+                        n_contrib, g2d, s_q, lo, hi, slot == kSegNone ? nullptr : seg.state(slot));
     }
 }
 
@@ -337,7 +337,7 @@ SegLayout frame_segments(const igs_frame& f) {
     if (f.tile != 16 && f.tile != 32) return SegLayout{};
     const SortScratch s = sort_scratch(f);
     const int64_t sub = f.tile / 8;
-    return seg_layout(s.seg_base, s.seg_bytes, (int64_t)f.tiles_x * f.tiles_y * sub * sub);
+    return seg_layout(s.seg_base, s.seg_bytes, s.seg_base2, s.seg_bytes2, (int64_t)f.tiles_x * f.tiles_y * sub * sub);
 }
 
 cudaError_t launch_blend_fwd(const igs_frame& f, const BlendParams& bp, float* img, cudaStream_t st, float* clear_g2d) {

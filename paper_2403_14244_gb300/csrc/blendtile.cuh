@@ -1,6 +1,6 @@
-// Per-tile front-to-back compositing (Eq. 4), shared by the one-view forward
-// kernel (blend.cu) and the persistent multi-view kernel (batch.cu), so both
-// produce bit-identical pixels. Internal to libigs.
+// Front-to-back compositing (Eq. 4), shared by the one-view forward kernel
+// (blend.cu) and the multi-view kernels (batch.cu), so all produce bit-identical
+// pixels. Internal to libigs.
 #pragma once
 
 #include "common.cuh"
@@ -37,47 +37,20 @@ __device__ __forceinline__ bool may_reach(float4 a, float xlo, float xhi, float 
     return !(eval_dist(cx, cy, a).pw > a.w);
 }
 
-// Block-wide last blend (max of last, +1 positions) into *s_hi of the caller's
-// shared memory.
-__device__ __forceinline__ void seg_reduce_into(uint32_t last, int lane, uint32_t* s_hi) {
-    const uint32_t whi = __reduce_max_sync(0xffffffffu, last);
-    if (lane == 0) atomicMax(s_hi, whi);
-}
-
 // One CTA of TS*TS threads composites one tile (one thread per pixel), staging
 // B entries at a time in shared memory (s_a, s_c hold B float4 each), and leaves
 // the batch loop once every pixel has stopped. Each warp owns an 8 x 4 block of
 // the tile (compact blocks are reached by fewer entries than whole rows, and
 // their pixels stop at similar depths) and walks, in order, only the staged
 // entries that may reach it (one ballot per 32 entries). Writes img (planar,
-// `plane` floats per channel, row stride `width`) and, if given, T_final /
-// n_contrib. SEG (one 8 x 8 block per CTA): the walk is cut into segments for
-// the backward (SegLayout), `block` naming this block.
-template <int TS, int B, bool SEG = false>
+// `plane` floats per channel, row stride `width`). The batch path's persistent
+// blend; pixels are bit for bit those of blend_block_fwd.
+template <int TS, int B>
 __device__ __forceinline__ void blend_tile_fwd(int tx, int ty, int width, int height, uint2 rg,
                                                const uint32_t* __restrict__ vals, const float4* __restrict__ rec,
                                                float alpha_min, float alpha_max, float t_min, const float* bg,
-                                               float4* s_a, float4* s_c, float* __restrict__ img,
-                                               float* __restrict__ T_final, uint32_t* __restrict__ n_contrib,
-                                               const SegLayout seg = SegLayout{}, uint32_t block = 0) {
+                                               float4* s_a, float4* s_c, float* __restrict__ img) {
     constexpr int NT = TS * TS;
-    static_assert(!SEG || NT == 64, "segments are cut per 8 x 8 block, one thread per pixel");
-    // segment state: where the open segment starts (the last cut), the block's
-    // last blend, and the slots of the segments closed so far
-    __shared__ uint32_t s_lo, s_hi, s_slot, s_n, s_stop;
-    __shared__ uint32_t s_slots[SEG ? kSegMaxPerBlock : 1];
-    uint32_t reserved = kSegNone;  // thread 0: the pool slot taken for the next close (its atomic
-                                   // is in flight meanwhile, off the block's path)
-    const bool segs = SEG && seg.slots != 0;
-    if (segs) {
-        if (threadIdx.x == 0) {
-            s_lo = 0;
-            s_hi = 0;
-            s_n = 0;
-            s_stop = 0;
-        }
-        __syncthreads();
-    }
     constexpr int BPR = TS / 8;  // 8 x 4 warp blocks per block row of the tile
     static_assert(B <= NT, "staging batch larger than the tile");
     static_assert(TS >= 8 && TS <= 32, "the tile holds whole 8 x 4 warp blocks");
@@ -90,7 +63,6 @@ __device__ __forceinline__ void blend_tile_fwd(int tx, int ty, int width, int he
     const float bx0 = (float)bx + 0.5f, bx1 = bx0 + 7.f;
     const float by0 = (float)by + 0.5f, by1 = by0 + 3.f;
     float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-    uint32_t last = 0;
     bool done = !inside;
     // Software-pipelined staging: thread t < B stages entry b0 + t of every
     // batch, its ids fetched two batches ahead and its records one batch ahead,
@@ -109,39 +81,6 @@ __device__ __forceinline__ void blend_tile_fwd(int tx, int ty, int width, int he
     }
     for (uint32_t b0 = rg.x; b0 < rg.y; b0 += B) {
         if (__syncthreads_count(done) == NT) break;
-        if constexpr (SEG) {
-            const uint32_t P = b0 - rg.x;
-            if (segs && P > 0 && P % kSegStride == 0) {
-                // close the open segment here if it holds blends: each pixel's state is
-                // that after every entry before P (its colour is turned into the colour
-                // behind once the walk has ended)
-                seg_reduce_into(last, lane, &s_hi);
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    uint32_t slot = kSegNone;
-                    if (s_hi > s_lo && !s_stop && s_n < kSegMaxPerBlock) {  // blends since the last cut
-                        if (reserved == kSegNone) {  // first close: this slot and the next one
-                            slot = atomicAdd(&seg.ctrl->slots_used, 2u);
-                            reserved = slot + 1;
-                        } else {
-                            slot = reserved;
-                            reserved = atomicAdd(&seg.ctrl->slots_used, 1u);
-                        }
-                        if (slot >= seg.slots) {
-                            slot = kSegNone;
-                            s_stop = 1;  // pool full: the block's last segment takes the rest
-                        } else {
-                            seg.items[slot] = make_uint4(block, s_lo, s_hi, slot);
-                            s_slots[s_n++] = slot;
-                            s_lo = P;
-                        }
-                    }
-                    s_slot = slot;
-                }
-                __syncthreads();
-                if (s_slot != kSegNone) seg.pool[(size_t)s_slot * 64 + threadIdx.x] = make_float4(T, C0, C1, C2);
-            }
-        }
         if (stager) {
             const uint32_t j = b0 + threadIdx.x;
             if (j < rg.y) {
@@ -179,27 +118,6 @@ __device__ __forceinline__ void blend_tile_fwd(int tx, int ty, int width, int he
                 C1 = fmaf(c.y, w, C1);
                 C2 = fmaf(c.z, w, C2);
                 T = Tn;
-                last = b0 - rg.x + k + 1;
-            }
-        }
-    }
-    if constexpr (SEG) {
-        if (segs) {
-            seg_reduce_into(last, lane, &s_hi);
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                // (no segment closed: the last segment is the whole walk; lo = kSegNone:
-                // no blend after the last cut)
-                seg.last[block] = s_n == 0 ? make_uint4(0u, 0u, kSegNone, 0u)
-                                           : make_uint4(s_n, s_hi > s_lo ? s_lo : kSegNone, s_hi, 0u);
-                if (reserved != kSegNone && reserved < seg.slots)
-                    seg.items[reserved] = make_uint4(kSegNone, 0u, 0u, kSegNone);  // taken, not used
-            }
-            // the saved colours become the colour composited behind each cut
-            for (uint32_t i = 0; i < s_n; ++i) {
-                float4* q = seg.pool + (size_t)s_slots[i] * 64 + threadIdx.x;
-                const float4 v = *q;
-                *q = make_float4(v.x, fmaf(T, bg[0], C0 - v.y), fmaf(T, bg[1], C1 - v.z), fmaf(T, bg[2], C2 - v.w));
             }
         }
     }
@@ -208,8 +126,6 @@ __device__ __forceinline__ void blend_tile_fwd(int tx, int ty, int width, int he
     img[pix] = fmaf(T, bg[0], C0);
     img[plane + pix] = fmaf(T, bg[1], C1);
     img[2 * plane + pix] = fmaf(T, bg[2], C2);
-    if (T_final) T_final[pix] = T;
-    if (n_contrib) n_contrib[pix] = last;
 }
 
 // ---- one warp per 8 x 8 pixel block ----
@@ -294,34 +210,56 @@ struct FwdPixels {
     float2 T;
     float2 thr;        // alpha threshold: alpha_min, or infinity once stopped
     float C[2][3];
+    float D[2][3];     // colour composited since the last cut (walk segments, after the first cut)
     uint32_t last[2];  // last blended list position + 1
 };
 
 // One pixel of a pair: blend the entry with the given alpha, T (1 - alpha) and
 // alpha T, by the comparisons of Eq. 4's rules in their order (skip, stop, blend),
 // as predicated instructions: nothing is added where the entry is not blended.
+// SUM: the entry's colour is added to D too.
+template <bool SUM>
 __device__ __forceinline__ void fwd_blend_one(float npw, float npmax, float alpha, float Tn, float w, const float4& c,
                                               uint32_t pos1, float t_min, float& T, float& thr, float (&C)[3],
-                                              uint32_t& last) {
-    asm("{\n\t"
-        ".reg .pred near, in, stop, go;\n\t"
-        "setp.geu.f32 near, %6, %7;\n\t"                // !(w2 d^2 > pmax)
-        "setp.ge.and.f32 in, %8, %1, near;\n\t"         // alpha >= threshold
-        "setp.lt.and.f32 stop|go, %9, %15, in;\n\t"     // T (1 - alpha) < t_min, or blended
-        "@stop mov.f32 %1, 0f7F800000;\n\t"
-        "@go fma.rn.f32 %2, %11, %10, %2;\n\t"
-        "@go fma.rn.f32 %3, %12, %10, %3;\n\t"
-        "@go fma.rn.f32 %4, %13, %10, %4;\n\t"
-        "@go mov.f32 %0, %9;\n\t"
-        "@go mov.u32 %5, %14;\n\t"
-        "}"
-        : "+f"(T), "+f"(thr), "+f"(C[0]), "+f"(C[1]), "+f"(C[2]), "+r"(last)
-        : "f"(npw), "f"(npmax), "f"(alpha), "f"(Tn), "f"(w), "f"(c.x), "f"(c.y), "f"(c.z), "r"(pos1), "f"(t_min));
+                                              float (&D)[3], uint32_t& last) {
+    if constexpr (SUM)
+        asm("{\n\t"
+            ".reg .pred near, in, stop, go;\n\t"
+            "setp.geu.f32 near, %9, %10;\n\t"             // !(w2 d^2 > pmax)
+            "setp.ge.and.f32 in, %11, %1, near;\n\t"      // alpha >= threshold
+            "setp.lt.and.f32 stop|go, %12, %18, in;\n\t"  // T (1 - alpha) < t_min, or blended
+            "@stop mov.f32 %1, 0f7F800000;\n\t"
+            "@go fma.rn.f32 %2, %14, %13, %2;\n\t"
+            "@go fma.rn.f32 %3, %15, %13, %3;\n\t"
+            "@go fma.rn.f32 %4, %16, %13, %4;\n\t"
+            "@go fma.rn.f32 %6, %14, %13, %6;\n\t"
+            "@go fma.rn.f32 %7, %15, %13, %7;\n\t"
+            "@go fma.rn.f32 %8, %16, %13, %8;\n\t"
+            "@go mov.f32 %0, %12;\n\t"
+            "@go mov.u32 %5, %17;\n\t"
+            "}"
+            : "+f"(T), "+f"(thr), "+f"(C[0]), "+f"(C[1]), "+f"(C[2]), "+r"(last), "+f"(D[0]), "+f"(D[1]), "+f"(D[2])
+            : "f"(npw), "f"(npmax), "f"(alpha), "f"(Tn), "f"(w), "f"(c.x), "f"(c.y), "f"(c.z), "r"(pos1), "f"(t_min));
+    else
+        asm("{\n\t"
+            ".reg .pred near, in, stop, go;\n\t"
+            "setp.geu.f32 near, %6, %7;\n\t"
+            "setp.ge.and.f32 in, %8, %1, near;\n\t"
+            "setp.lt.and.f32 stop|go, %9, %15, in;\n\t"
+            "@stop mov.f32 %1, 0f7F800000;\n\t"
+            "@go fma.rn.f32 %2, %11, %10, %2;\n\t"
+            "@go fma.rn.f32 %3, %12, %10, %3;\n\t"
+            "@go fma.rn.f32 %4, %13, %10, %4;\n\t"
+            "@go mov.f32 %0, %9;\n\t"
+            "@go mov.u32 %5, %14;\n\t"
+            "}"
+            : "+f"(T), "+f"(thr), "+f"(C[0]), "+f"(C[1]), "+f"(C[2]), "+r"(last)
+            : "f"(npw), "f"(npmax), "f"(alpha), "f"(Tn), "f"(w), "f"(c.x), "f"(c.y), "f"(c.z), "r"(pos1), "f"(t_min));
 }
 
 // Walk U queued entries from e on: their alphas first (independent of one
 // another), then the pixels' transmittances entry by entry.
-template <int U>
+template <int U, bool SUM>
 __device__ __forceinline__ void fwd_walk_some(const FwdEntry* e, float alpha_max, float t_min, FwdPixels& s) {
     float2 npw[U], alpha[U], oma[U];
     float4 c[U];
@@ -343,10 +281,10 @@ __device__ __forceinline__ void fwd_walk_some(const FwdEntry* e, float alpha_max
 #pragma unroll
     for (int k = 0; k < U; ++k) {
         const float2 Tn = pk_mul(s.T, oma[k]), w = pk_mul(alpha[k], s.T);
-        fwd_blend_one(npw[k].x, npmax[k], alpha[k].x, Tn.x, w.x, c[k], pos1[k], t_min, s.T.x, s.thr.x, s.C[0],
-                      s.last[0]);
-        fwd_blend_one(npw[k].y, npmax[k], alpha[k].y, Tn.y, w.y, c[k], pos1[k], t_min, s.T.y, s.thr.y, s.C[1],
-                      s.last[1]);
+        fwd_blend_one<SUM>(npw[k].x, npmax[k], alpha[k].x, Tn.x, w.x, c[k], pos1[k], t_min, s.T.x, s.thr.x, s.C[0],
+                           s.D[0], s.last[0]);
+        fwd_blend_one<SUM>(npw[k].y, npmax[k], alpha[k].y, Tn.y, w.y, c[k], pos1[k], t_min, s.T.y, s.thr.y, s.C[1],
+                           s.D[1], s.last[1]);
     }
 }
 
@@ -354,12 +292,13 @@ __device__ __forceinline__ void fwd_walk_some(const FwdEntry* e, float alpha_max
 // independent work between two steps of the transmittance chain, which is what a
 // long walk waits for once few warps are left (two and eight measured alike, within 1 %).
 constexpr int kFwdUnroll = 4;
+template <bool SUM>
 __device__ __forceinline__ void fwd_walk(const FwdEntry* e, int cnt, float alpha_max, float t_min, FwdPixels& s) {
     int k = 0;
 #pragma unroll 1
-    for (; k + kFwdUnroll <= cnt; k += kFwdUnroll) fwd_walk_some<kFwdUnroll>(e + k, alpha_max, t_min, s);
+    for (; k + kFwdUnroll <= cnt; k += kFwdUnroll) fwd_walk_some<kFwdUnroll, SUM>(e + k, alpha_max, t_min, s);
 #pragma unroll 1
-    for (; k < cnt; ++k) fwd_walk_some<1>(e + k, alpha_max, t_min, s);
+    for (; k < cnt; ++k) fwd_walk_some<1, SUM>(e + k, alpha_max, t_min, s);
 }
 
 // One warp composites the 8 x 8 block at pixel (bx, by), walking the tile's
@@ -387,7 +326,7 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
     s.T = make_float2(1.f, 1.f);
     s.thr = make_float2(x < width && y0 < height ? alpha_min : inf, x < width && y1 < height ? alpha_min : inf);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) s.C[i][0] = s.C[i][1] = s.C[i][2] = 0.f;
+    for (int i = 0; i < 2; ++i) s.C[i][0] = s.C[i][1] = s.C[i][2] = s.D[i][0] = s.D[i][1] = s.D[i][2] = 0.f;
     s.last[0] = s.last[1] = 0;
     // segment state (warp-uniform): where the open segment starts (the last cut), the segments closed
     uint32_t seg_lo = 0, seg_n = 0;
@@ -399,8 +338,13 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
     auto walk = [&](uint32_t cnt) {  // the first cnt queued entries; whether every pixel has stopped
         __syncwarp();
         const uint32_t first = min(cnt, kQueue - head);
-        fwd_walk(Q.e + head, (int)first, alpha_max, t_min, s);
-        if (first < cnt) fwd_walk(Q.e, (int)(cnt - first), alpha_max, t_min, s);
+        if (SEG && seg_n > 0) {  // past the first cut: the open segment's own colour too
+            fwd_walk<true>(Q.e + head, (int)first, alpha_max, t_min, s);
+            if (first < cnt) fwd_walk<true>(Q.e, (int)(cnt - first), alpha_max, t_min, s);
+        } else {
+            fwd_walk<false>(Q.e + head, (int)first, alpha_max, t_min, s);
+            if (first < cnt) fwd_walk<false>(Q.e, (int)(cnt - first), alpha_max, t_min, s);
+        }
         queued -= cnt;
         head = queued ? (head + cnt) & (kQueue - 1) : 0u;
         return __all_sync(0xffffffffu, s.thr.x == inf && s.thr.y == inf);  // (also: the entries may be overwritten)
@@ -409,10 +353,11 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
     for (uint32_t b = 0; b * 32 < n && !done; ++b) {
         const uint32_t b0 = b * 32;
         if constexpr (SEG) {
-            if (segs && b0 > 0 && b0 % kSegStride == 0) {
+            if (segs && b0 > 0 && (b0 & (seg.stride - 1)) == 0) {
                 if (queued && walk(queued)) break;
-                // close the open segment here if it holds blends: each pixel's state is that after
-                // every entry before b0 (its colour is turned into the colour behind once the walk has ended)
+                // close the open segment here if it holds blends: each pixel's T is that after every
+                // entry before b0, and the segment's own colour is kept until the walk has ended and
+                // the colour behind the cut can be summed
                 const uint32_t hi = __reduce_max_sync(0xffffffffu, max(s.last[0], s.last[1]));
                 if (hi > seg_lo && !seg_stop && seg_n < kSegMaxPerBlock) {
                     uint32_t pool_slot = 0;
@@ -433,11 +378,14 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
                             seg.items[pool_slot] = make_uint4(block, seg_lo, hi, pool_slot);
                             Q.slots[seg_n] = pool_slot;
                         }
+                        const float(&own)[2][3] = seg_n == 0 ? s.C : s.D;  // the first segment's colour is all there is
+                        float4* st = seg.state(pool_slot) + lane;
+                        st[0] = make_float4(s.T.x, own[0][0], own[0][1], own[0][2]);
+                        st[32] = make_float4(s.T.y, own[1][0], own[1][1], own[1][2]);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) s.D[i][0] = s.D[i][1] = s.D[i][2] = 0.f;
                         ++seg_n;
                         seg_lo = b0;
-                        float4* st = seg.pool + (size_t)pool_slot * 64 + lane;
-                        st[0] = make_float4(s.T.x, s.C[0][0], s.C[0][1], s.C[0][2]);
-                        st[32] = make_float4(s.T.y, s.C[1][0], s.C[1][1], s.C[1][2]);
                     }
                 }
             }
@@ -473,15 +421,26 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
                     seg.items[reserved] = make_uint4(kSegNone, 0u, 0u, kSegNone);  // taken, not used
             }
             __syncwarp();
-            // the saved colours become the colour composited behind each cut
-            for (uint32_t i = 0; i < seg_n; ++i) {
-                float4* st = seg.pool + (size_t)Q.slots[i] * 64 + lane;
+            // the saved colours become the colour composited behind each cut: the background through
+            // the last segment's T and the segments behind the cut, from the back (as the difference
+            // of the colours up to the end and up to the cut, the little that shines through from
+            // behind a nearly opaque front would keep few of its digits)
+            if (seg_n > 0) {
+                float S[2][3];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float4 v = st[32 * h];
-                    const float T = h ? s.T.y : s.T.x;
-                    st[32 * h] = make_float4(v.x, fmaf(T, bg[0], s.C[h][0] - v.y), fmaf(T, bg[1], s.C[h][1] - v.z),
-                                             fmaf(T, bg[2], s.C[h][2] - v.w));
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) S[h][ch] = fmaf(h ? s.T.y : s.T.x, bg[ch], s.D[h][ch]);
+                for (uint32_t i = seg_n; i-- > 0;) {
+                    float4* st = seg.state(Q.slots[i]) + lane;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 v = st[32 * h];
+                        st[32 * h] = make_float4(v.x, S[h][0], S[h][1], S[h][2]);
+                        S[h][0] += v.y;
+                        S[h][1] += v.z;
+                        S[h][2] += v.w;
+                    }
                 }
             }
         }

@@ -323,7 +323,9 @@ struct SortScratch {
     uint2* walk_rect;                 // [n] rectangle of order[p] (level-1 count writes, level-1 place reads)
     uint32_t* tile_order;             // [tiles] tiles by descending entry count, for the blends; nullptr: as they come
     void* seg_base;                   // the depth items' buffers (ditems_a, ditems_b), reused by the blends'
-    size_t seg_bytes;                 // walk segments once binning is done
+    size_t seg_bytes;                 // walk segments once binning is done,
+    void* seg_base2;                  // and the level-1 counts, for more of their pool
+    size_t seg_bytes2;
     int64_t walk_chunks;              // > 0: counting sort of the entries; 0: duplication + tile radix passes
     int tile_passes;
     int tile_bits;
@@ -342,22 +344,29 @@ cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStrea
 size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t tiles_y, int64_t chunks);
 
 // Walk segments of the one-view blends (16- and 32-pixel binning tiles, one
-// 8 x 8 pixel block per CTA). A block whose walk is long closes a segment at
-// a list position that is a multiple of kSegStride when the open segment holds
+// 8 x 8 pixel block per warp). A block whose walk is long closes a segment at
+// a list position that is a multiple of `stride` when the open segment holds
 // blends: it saves each pixel's state there (T, and the colour composited
 // behind that position, once the walk has ended) in a pool slot, so that the
 // backward can walk every segment in parallel instead of one block walking its
 // whole list. A closed segment is items[slot] = (block, lo, hi, slot): list
 // positions relative to the tile's first entry, lo = the cut it starts at, hi =
-// one past its last blend, the state at hi in pool[slot]; a slot taken but not used
-// holds block = kSegNone. A block's last segment, which ends with the final
+// one past its last blend, the state at hi in slot's pixels; a slot taken but not
+// used holds block = kSegNone. A block's last segment, which ends with the final
 // state (T_final and the background), is last[block] = (segments closed, lo,
-// hi, -); lo = kSegNone when it holds no blend. The pieces live in the frame's
-// depth-sort item buffers, which binning no longer needs once the entries are
-// placed.
-constexpr uint32_t kSegStride = 1024;        // list positions; a multiple of the forward's 64-entry batches
+// hi, -); lo = kSegNone when it holds no blend. The pieces live in scratch that
+// binning no longer needs once the entries are placed: the depth-sort item
+// buffers and the level-1 counts.
 constexpr uint32_t kSegNone = 0xFFFFFFFFu;
 constexpr int kSegMaxPerBlock = 64;          // segments a block closes at most (the rest stay in its last one)
+// List positions between cuts, multiples of the blends' 32-entry batches. A frame of few blocks leaves
+// most of the backward's warps without work, and its time is that of the longest piece: with cuts every
+// 256 positions instead of 1024, the training step of 30,000 Gaussians at 401 x 299 pixels (1976 blocks,
+// walks up to 870) takes 147 us instead of 175 (512: 172). With many blocks the cuts gain the backward
+// about 1 % (3M training step 1340 -> 1326 us) and cost a forward without a backward up to 4 % (200,000
+// Gaussians at 1001 x 667, 10584 blocks: 190 -> 199 us), so those keep 1024.
+constexpr uint32_t kSegStride = 1024, kSegStrideFew = 256;
+constexpr int64_t kSegFewBlocks = 8192;
 struct SegCtrl {                             // all zeroed before each forward; next (the
     uint32_t next, slots_used, pad0, pad1;   // backward's work counter) also before each backward
 };
@@ -365,25 +374,38 @@ struct SegLayout {
     SegCtrl* ctrl;
     uint4* last;      // [blocks] (closed, lo, hi, -) of each block's last segment
     uint4* items;     // [slots] (block, lo, hi, slot) of each closed segment
-    float4* pool;     // [slots][64] (T, S_r, S_g, S_b) per pixel of the block, pixel = row * 8 + column
+    float4* pool;     // [slots][64] (T, S_r, S_g, S_b) per pixel of the block, pixel = row * 8 + column:
+    float4* pool2;    // slots below `split` in pool, the others in pool2
+    uint32_t split;
     uint32_t slots;   // 0: segments off
     uint32_t blocks;
+    uint32_t stride;  // a power of two
+    __device__ __forceinline__ float4* state(uint32_t slot) const {
+        return slot < split ? pool + (size_t)slot * 64 : pool2 + (size_t)(slot - split) * 64;
+    }
 };
-// Carved from [base, base + bytes) for `blocks` 8 x 8 blocks (slots = 0 when it does not fit).
-__host__ __device__ inline SegLayout seg_layout(void* base, size_t bytes, int64_t blocks) {
+// Carved for `blocks` 8 x 8 blocks: everything but the second part of the pool from [base, base + bytes),
+// that from [base2, base2 + bytes2) (slots = 0 when the first does not hold it).
+__host__ __device__ inline SegLayout seg_layout(void* base, size_t bytes, void* base2, size_t bytes2, int64_t blocks) {
     SegLayout L{};
     const size_t head = 256 + (((size_t)blocks * 16 + 255) & ~(size_t)255);
-    if (!base || bytes < head + 1040 || blocks <= 0 || blocks >= (1 << 24)) return L;
-    int64_t slots = (int64_t)((bytes - head) / 1040);  // 16 B item + 1 KB of pixel states per slot
-    if (slots > (1 << 20)) slots = 1 << 20;
+    if (!base || blocks <= 0 || blocks >= (1 << 24)) return L;
+    size_t more = base2 ? bytes2 / 1024 : 0;  // slots of the second part
+    if (more > (1 << 19)) more = 1 << 19;
+    if (bytes < head + 1040 + 512 + 16 * more) more = 0;
+    if (bytes < head + 1040 + 512) return L;
+    int64_t slots = (int64_t)((bytes - head - 512 - 16 * more) / 1040);  // 16 B item + 1 KB of pixel states per slot
+    if (slots > (1 << 19)) slots = 1 << 19;
     char* p = static_cast<char*>(base);
     L.ctrl = reinterpret_cast<SegCtrl*>(p);
     L.last = reinterpret_cast<uint4*>(p + 256);
     L.items = reinterpret_cast<uint4*>(p + head);
-    L.pool = reinterpret_cast<float4*>(p + head + (((size_t)slots * 16 + 255) & ~(size_t)255));
-    if ((size_t)(reinterpret_cast<char*>(L.pool) - p) + (size_t)slots * 1024 > bytes) --slots;
-    L.slots = slots > 0 ? (uint32_t)slots : 0;
+    L.pool = reinterpret_cast<float4*>(p + head + ((16 * ((size_t)slots + more) + 255) & ~(size_t)255));
+    L.pool2 = static_cast<float4*>(base2);
+    L.split = (uint32_t)slots;
+    L.slots = (uint32_t)(slots + (int64_t)more);
     L.blocks = (uint32_t)blocks;
+    L.stride = blocks <= kSegFewBlocks ? kSegStrideFew : kSegStride;
     return L;
 }
 int64_t sort_walk_chunks(int64_t tiles_x, int64_t tiles_y);

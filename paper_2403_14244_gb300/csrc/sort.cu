@@ -1033,6 +1033,8 @@ SortScratch sort_scratch(const igs_frame& f) {
     s.grid = (int32_t*)take((size_t)(2 * tiles + 2 + f.tiles_y + 1) * 4);
     const int64_t rows = chunks > 0 ? f.tiles_y : 0;
     s.walk_h1 = (uint32_t*)take((size_t)chunks * rows * 4);
+    s.seg_base2 = chunks > 0 ? s.walk_h1 : nullptr;
+    s.seg_bytes2 = (size_t)chunks * rows * 4;
     s.walk_len = (uint32_t*)take((size_t)rows * 4);
     s.walk_rows = (uint32_t*)take((size_t)(3 * rows + 1) * 4);
     s.walk_h2 = (uint32_t*)take((size_t)(chunks > 0 ? l2_chunks_max(cap, f.tiles_y) * f.tiles_x : 0) * 4);
