@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(kSsimThreads) k_ssim_fwd(const float* __restri
                                                           SsimParams P, float2* __restrict__ mAB,
                                                           float* __restrict__ mC, float* __restrict__ loss,
                                                           float* __restrict__ ssim) {
+    pdl_wait();
     __shared__ SsimFwdSmem sm;
     const int W = P.width, H = P.height;
     const size_t plane = (size_t)W * H, base = (size_t)blockIdx.z * plane;
@@ -216,6 +217,7 @@ struct SsimBwdSmem {
 __global__ void __launch_bounds__(kSsimThreads) k_ssim_bwd(const float* __restrict__ img, const float* __restrict__ target,
                                                           const float2* __restrict__ mAB, const float* __restrict__ mC,
                                                           SsimParams P, float* __restrict__ grad) {
+    pdl_wait();
     __shared__ SsimBwdSmem sm;
     const int W = P.width, H = P.height;
     const size_t plane = (size_t)W * H, base = (size_t)blockIdx.z * plane;
@@ -297,18 +299,25 @@ cudaError_t launch_l1_ssim(const float* img, const float* target, int channels, 
     P.s_scale = (float)(lambda / count);
     P.lambda = lambda;
     P.inv_count = (float)(1.0 / count);
-    cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
-    if (e == cudaSuccess && ssim) e = cudaMemsetAsync(ssim, 0, sizeof(float), st);
+    // both sums cleared in one launch of the chain (memsets between its kernels would drain it)
+    ZeroRanges z = {};
+    for (float* p : {loss, ssim})
+        if (p) {
+            z.ptr[z.count] = p;
+            z.bytes[z.count++] = sizeof(float);
+        }
+    cudaError_t e = launch_zero(z, st);
     if (e != cudaSuccess) return e;
     const size_t count_e = (size_t)channels * height * width;
     float2* mAB = reinterpret_cast<float2*>(work);  // (A, B) pairs, then C
     float* mC = work + 2 * count_e;
     const dim3 grid((unsigned)ceil_div(width, kSsimTile), (unsigned)ceil_div(height, kSsimTile), (unsigned)channels);
-    k_ssim_fwd<<<grid, kSsimThreads, 0, st>>>(img, target, P, mAB, mC, loss, ssim);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_ssim_bwd<<<grid, kSsimThreads, 0, st>>>(img, target, mAB, mC, P, grad);
+    if ((e = launch_pdl(k_ssim_fwd, grid, dim3(kSsimThreads), 0, st, img, target, P, mAB, mC, loss, ssim)) != cudaSuccess)
+        return e;
+    e = launch_pdl(k_ssim_bwd, grid, dim3(kSsimThreads), 0, st, img, target, (const float2*)mAB, (const float*)mC, P,
+                   grad);
     count_launches(2);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace igs
