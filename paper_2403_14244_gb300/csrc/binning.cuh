@@ -104,13 +104,14 @@ __global__ void __launch_bounds__(1024) k_hist_to_offsets(uint32_t* __restrict__
 // SKIPPABLE (one segment only): when *skip_flag is set, the pass writes only
 // the values, to skip_vals, or, without skip_vals, does nothing (the redundant
 // top pass of a depth sort whose third pass wrote the order).
-template <bool IN_KEYS32, bool OUT_VALS, bool SKIPPABLE = false>
+template <bool IN_KEYS32, bool OUT_VALS, bool SKIPPABLE = false, int IPT = kSortIpt>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     const void* __restrict__ in_, void* __restrict__ out_, const uint32_t* __restrict__ d_count, uint32_t count_host,
     int shift, const uint32_t* __restrict__ digit_base, uint32_t* __restrict__ status,
     uint32_t* __restrict__ block_counter, uint32_t* __restrict__ info, uint32_t silent_blk = 0xFFFFFFFFu,
     const uint32_t* __restrict__ skip_flag = nullptr, uint32_t* __restrict__ skip_vals = nullptr) {
     pdl_wait();
+    constexpr int kTile = kSortThreads * IPT;  // items per block
     if (SKIPPABLE && !skip_vals && *skip_flag) return;
     {
         const uint64_t seg = blockIdx.y;
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
         block_counter += seg;
     }
     const uint64_t seg_base = (uint64_t)blockIdx.y * count_host;
-    __shared__ u64 s_items[kSortTile];
+    __shared__ u64 s_items[kTile];
     __shared__ uint16_t s_whist[kWarps][kRadix];  // per warp: running count, then block-local start
     __shared__ uint32_t s_cnt[kRadix];
     __shared__ int32_t s_delta[kRadix];           // global position - staged position, per digit
@@ -146,16 +147,16 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     }
     __syncthreads();
     const uint32_t blk = s_blk;
-    const uint64_t base = (uint64_t)blk * kSortTile;
+    const uint64_t base = (uint64_t)blk * kTile;
     if (base >= count) return;  // no later block depends on a block past the end
-    const uint32_t valid = (uint32_t)min((uint64_t)kSortTile, (uint64_t)count - base);
+    const uint32_t valid = (uint32_t)min((uint64_t)kTile, (uint64_t)count - base);
 
     // warp-striped load: warp w owns [w*32*IPT, (w+1)*32*IPT), item i of lane l is i*32 + l
-    u64 it[kSortIpt];
-    const uint32_t wbase = w * 32 * kSortIpt + lane;
-    if (valid == kSortTile) {
+    u64 it[IPT];
+    const uint32_t wbase = w * 32 * IPT + lane;
+    if (valid == kTile) {
 #pragma unroll
-        for (int i = 0; i < kSortIpt; ++i) {
+        for (int i = 0; i < IPT; ++i) {
             const uint64_t g = base + wbase + i * 32;
             if (IN_KEYS32)
                 it[i] = ((u64)static_cast<const uint32_t*>(in_)[g] << 32) | (uint32_t)(seg_base + g);
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kSortIpt; ++i) {
+        for (int i = 0; i < IPT; ++i) {
             const uint32_t loc = wbase + i * 32;
             const uint64_t g = base + loc;
             if (loc < valid)
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     }
     // digit counts of the block's valid items, published before the ranking
 #pragma unroll
-    for (int i = 0; i < kSortIpt; ++i)
+    for (int i = 0; i < IPT; ++i)
         if (wbase + i * 32 < valid) atomicAdd(&s_cnt[(uint32_t)(it[i] >> (32 + shift)) & 0xFFu], 1u);
     __syncthreads();
     uint32_t* my = status + (size_t)blk * kRadix;
@@ -185,10 +186,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     const bool silent = blk == silent_blk;
     if (!silent) st_relaxed_u32(&my[tid], (blk == 0 ? kFlagPre : kFlagAgg) | (s_cnt[tid] & kValMask));
     // rank within the warp, in item order
-    uint32_t rank2[kSortIpt / 2];  // two 16-bit ranks per register (ranks < kSortTile)
+    uint32_t rank2[IPT / 2];  // two 16-bit ranks per register (ranks < kTile)
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
-    for (int i = 0; i < kSortIpt; ++i) {
+    for (int i = 0; i < IPT; ++i) {
         const uint32_t d = (uint32_t)(it[i] >> (32 + shift)) & 0xFFu;
         // peers: lanes with the same digit, from 8 ballots (measured faster than match.any here)
         uint32_t peers = 0xffffffffu;
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     // stage the block's items in digit order (needs only block-local offsets, so it
     // runs before the look-back and gives earlier blocks time to publish)
 #pragma unroll
-    for (int i = 0; i < kSortIpt; ++i) {
+    for (int i = 0; i < IPT; ++i) {
         const uint32_t d = (uint32_t)(it[i] >> (32 + shift)) & 0xFFu;
         s_items[s_whist[w][d] + ((rank2[i >> 1] >> (16 * (i & 1))) & 0xFFFFu)] = it[i];
     }
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     __syncthreads();
     // write out: runs of one digit land contiguously; past-the-end items hold the last slots
 #pragma unroll
-    for (int k = 0; k < kSortIpt; ++k) {
+    for (int k = 0; k < IPT; ++k) {
         const uint32_t q = k * kSortThreads + tid;
         if (q >= valid) continue;
         const u64 item = s_items[q];

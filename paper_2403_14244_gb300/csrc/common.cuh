@@ -32,6 +32,14 @@ enum : int { kInfoM = 0, kInfoKept = 1, kInfoErr = 2, kInfoNeed = 3, kInfoAbort 
 constexpr int kSortThreads = 256;
 constexpr int kSortIpt = 20;
 constexpr int kSortTile = kSortThreads * kSortIpt;
+// Depth sorts of so few Gaussians that blocks of 5120 would not cover the SMs take 8 items
+// per thread: a pass is then a chain of latencies, and the ranking's share of it shrinks. (A frame of 200K: 177 us
+// with 20, 166 so; bursts of 500K frames 1 %; at 2M 8 items cost 2 to 5 %.)
+constexpr int kSortIptFew = 8;
+constexpr int64_t kSortFew = 152 * (int64_t)kSortTile;
+__host__ __device__ constexpr int64_t depth_sort_tile(int64_t n) {
+    return n <= kSortFew ? kSortThreads * kSortIptFew : kSortTile;
+}
 constexpr int kRadix = 256;
 constexpr int kScanThreads = 256;
 constexpr int kScanIpt = 16;

@@ -59,6 +59,13 @@ constexpr uint32_t kStage = 1536;          // staged entries per level-2 chunk
 constexpr uint32_t kChunkTarget = kStage * 4 / 5;
 constexpr uint32_t kStage1 = 768;          // staged 8-byte items per level-1 chunk
 constexpr uint32_t kChunkTarget1 = kStage1 * 4 / 5;
+// Chunks of a walk, at least (while they hold 32 items, level 2's 128 entries): a walk of fewer
+// chunks leaves SM schedulers idle, and a chunk is one warp's chain of dependent steps. With full
+// chunks a frame of 200K Gaussians and 1.2M entries has 500 and 1000. (A frame of 200K at
+// 1001 x 667: 182 us with full chunks, 166 so; with 1216 or 4864 chunks at least 174, and 4864
+// costs a frame of 1M 15 of 352.)
+constexpr uint32_t kWalkFill = 2432;
+constexpr uint32_t kChunkLeast = 128;
 constexpr int kWalkWarps = 4;              // warps per CTA of the walk kernels (one chunk each)
 constexpr int kWalkUnroll = 8;             // items per lane per round of the counting walks
 
@@ -210,8 +217,8 @@ __device__ __forceinline__ void publish_tile_total(unsigned long long* s_total, 
 // rectangle spans tile row y (prefix of the row differences rowd), the length
 // of row y's level-1 list. rowinfo = [rows] list starts (prefix of len),
 // [rows] first level-2 chunk, [rows] items per level-2 chunk, [1] level-2 chunk
-// total. A row's level-2 chunks take about kChunkTarget entries each:
-// kChunkTarget * len / entries items, at least 32, where the row's entries are
+// total. A row's level-2 chunks take about `target` entries each (kChunkTarget or fewer):
+// target * len / entries items, at least 32, where the row's entries are
 // rowstart[y + 1] - rowstart[y] (rowstart[y]: the first entry of the row's
 // tiles, held in column tiles_x of the grid g; rowstart[rows] = M). Records an
 // error if the chunks exceed max_chunks.
@@ -227,13 +234,18 @@ __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, con
     uint32_t dsum = 0;
     for (uint32_t y = y0; y < y1; ++y) dsum += (uint32_t)rowd[y];
     const uint32_t lfirst = block_excl_scan<NT>(dsum, s_warp);  // modulo 2^32: the differences' prefix
+    // entries per chunk: kChunkTarget, fewer where M has less than kWalkFill such chunks, as far as
+    // max_chunks allows: a row has at most 33/32 entries / target + 1 chunks (a chunk's items, 32 or
+    // more, are rounded down), so M / target <= 15/16 (max_chunks - rows) keeps their sum within it
+    const uint32_t fill = max(1u, min(kWalkFill, (max_chunks - min(max_chunks, rows)) / 16 * 15));
+    const uint32_t target = min(kChunkTarget, max(kChunkLeast, M / fill + 1));
     uint32_t items = 0, chunks = 0, run = lfirst;
     for (uint32_t y = y0; y < y1; ++y) {
         run += (uint32_t)rowd[y];
         const uint32_t ly = run;
         const uint64_t entries = rowstart(y + 1) - rowstart(y);
         const uint32_t size =
-            (uint32_t)max((uint64_t)32, entries ? (uint64_t)kChunkTarget * ly / entries : (uint64_t)kChunkTarget);
+            (uint32_t)max((uint64_t)32, entries ? (uint64_t)target * ly / entries : (uint64_t)target);
         len[y] = ly;
         rowinfo[2 * rows + y] = size;
         items += ly;
@@ -406,14 +418,15 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
 // Level-1 chunk c: positions [p0, p1) of the depth order among the kept
 // Gaussians; `used` chunks hold Gaussians. A chunk takes about kChunkTarget1 /
 // sqrt(M / kept) Gaussians (the rows of an isotropic footprint are about the
-// square root of its tiles).
+// square root of its tiles), fewer where the frame would have less than kWalkFill chunks.
 struct Chunk {
     uint32_t p0, p1, used;
 };
 __device__ __forceinline__ Chunk l1_chunk(uint32_t c, uint32_t cmax, const uint32_t* __restrict__ info) {
     const uint32_t kept = info[kInfoKept], M = info[kInfoM];
     const float rows_per = kept ? fmaxf(1.f, sqrtf((float)M / (float)kept)) : 1.f;
-    const uint32_t target = max(32u, (uint32_t)((float)kChunkTarget1 / rows_per));
+    const uint32_t target =
+        max(32u, min((uint32_t)((float)kChunkTarget1 / rows_per), (uint32_t)ceil_div(kept, kWalkFill)));
     const uint32_t per = max(target, (uint32_t)ceil_div(kept, cmax));
     Chunk ch;
     ch.used = (uint32_t)ceil_div(kept, per);
@@ -983,7 +996,7 @@ static bool orders_tiles(int64_t chunks, int64_t tiles) { return chunks > 0 && t
 // item buffers hold vals and tile_key.
 size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t tiles_y, int64_t chunks) {
     const int64_t tiles = tiles_x * tiles_y;
-    const int64_t bn = ceil_div(n, kSortTile), bc = ceil_div(capacity, kSortTile), bs = ceil_div(n, kScanTile);
+    const int64_t bn = ceil_div(n, depth_sort_tile(n)), bc = ceil_div(capacity, kSortTile), bs = ceil_div(n, kScanTile);
     const int tp = chunks > 0 ? 0 : tile_passes_for(tiles);
     const size_t entry = chunks > 0 ? 4 : 8;
     const int64_t rows = chunks > 0 ? tiles_y : 0;
@@ -1010,7 +1023,7 @@ size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t 
 SortScratch sort_scratch(const igs_frame& f) {
     SortScratch s;
     const int64_t n = f.n, cap = f.capacity, tiles = (int64_t)f.tiles_x * f.tiles_y;
-    const int64_t bn = ceil_div(n, kSortTile), bc = ceil_div(cap, kSortTile), bs = ceil_div(n, kScanTile);
+    const int64_t bn = ceil_div(n, depth_sort_tile(n)), bc = ceil_div(cap, kSortTile), bs = ceil_div(n, kScanTile);
     const int64_t chunks = f.sort_chunks;
     const size_t entry = chunks > 0 ? 4 : 8;
     s.tile_bits = tile_bits_for(tiles);
@@ -1055,11 +1068,47 @@ SortScratch sort_scratch(const igs_frame& f) {
 // with one silent block (igs_debug_silence_lookback_once).
 std::atomic<int> g_silence_next{0};
 
+// The four passes of a frame's depth sort (small_grid: k_tiles_small decides the top-pass skip).
+template <int IPT>
+static cudaError_t launch_depth_sort(const igs_frame& f, const SortScratch& s, bool small_grid, cudaStream_t st) {
+    const uint32_t nn = (uint32_t)f.n;
+    const int64_t bn = ceil_div(f.n, kSortThreads * IPT);
+    const dim3 blocks((unsigned)bn), threads(kSortThreads);
+    const uint32_t* skip = f.info + kInfoSkipTop;
+    for (int p = 0; p < 4; ++p) {
+        uint32_t* status = s.status_depth + (size_t)p * bn * kRadix;
+        const uint32_t* hist = s.hist + p * kRadix;
+        cudaError_t e;
+        if (p == 0)
+            e = launch_pdl(k_radix_pass<true, false, false, IPT>, blocks, threads, 0, st, f.depth_key, s.ditems_a, nullptr,
+                           nn, 0, hist, status, s.counters + 0, f.info, g_silence_next.exchange(0) ? 1u : 0xFFFFFFFFu,
+                           nullptr, nullptr);
+        else if (p == 1)
+            e = launch_pdl(k_radix_pass<false, false, false, IPT>, blocks, threads, 0, st, s.ditems_a, s.ditems_b, nullptr,
+                           nn, 8, hist, status, s.counters + 1, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+        else if (p == 2 && small_grid)  // writes the order itself when the top pass is skipped
+            e = launch_pdl(k_radix_pass<false, false, true, IPT>, blocks, threads, 0, st, s.ditems_b, s.ditems_a, nullptr,
+                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, skip, f.order);
+        else if (p == 2)
+            e = launch_pdl(k_radix_pass<false, false, false, IPT>, blocks, threads, 0, st, s.ditems_b, s.ditems_a, nullptr,
+                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+        else if (small_grid)  // nothing to do when the top pass is skipped
+            e = launch_pdl(k_radix_pass<false, true, true, IPT>, blocks, threads, 0, st, s.ditems_a, f.order, nullptr, nn,
+                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, skip, nullptr);
+        else
+            e = launch_pdl(k_radix_pass<false, true, false, IPT>, blocks, threads, 0, st, s.ditems_a, f.order, nullptr, nn,
+                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+        count_launches();
+        if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) {
     const SortScratch s = sort_scratch(f);
     const int64_t n = f.n, cap = f.capacity;
     const int64_t tiles = (int64_t)f.tiles_x * f.tiles_y;
-    const int64_t bn = ceil_div(n, kSortTile), bc = ceil_div(cap, kSortTile), bs = ceil_div(n, kScanTile);
+    const int64_t bn = ceil_div(n, depth_sort_tile(n)), bc = ceil_div(cap, kSortTile), bs = ceil_div(n, kScanTile);
     const int tp = s.tile_passes;
     const int gx = f.tiles_x + 1, gy = f.tiles_y + 1;
     cudaError_t e;
@@ -1123,32 +1172,8 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
     }
     // 1. depth sort: (depth_key, index) -> A -> B -> A -> order (or -> order after the third pass)
     const bool small_grid = (int64_t)gx * gy <= kGridSmemCells;  // k_tiles_small decides the top-pass skip
-    for (int p = 0; p < 4; ++p) {
-        uint32_t* status = s.status_depth + (size_t)p * bn * kRadix;
-        const uint32_t* hist = s.hist + p * kRadix;
-        if (p == 0)
-            CK(launch_pdl(k_radix_pass<true, false>, dim3((unsigned)bn), dim3(kSortThreads), 0, st, 
-                f.depth_key, s.ditems_a, nullptr, nn, 0, hist, status, s.counters + 0, f.info,
-                g_silence_next.exchange(0) ? 1u : 0xFFFFFFFFu, nullptr, nullptr));
-        else if (p == 3 && small_grid)  // nothing to do when the top pass is skipped (k_tiles_small decides)
-            CK(launch_pdl(k_radix_pass<false, true, true>, dim3((unsigned)bn), dim3(kSortThreads), 0, st, 
-                s.ditems_a, f.order, nullptr, nn, 24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu,
-                f.info + kInfoSkipTop, nullptr));
-        else if (p == 3)
-            CK(launch_pdl(k_radix_pass<false, true>, dim3((unsigned)bn), dim3(kSortThreads), 0, st, 
-                s.ditems_a, f.order, nullptr, nn, 24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu,
-                nullptr, nullptr));
-        else if (p == 2 && small_grid)  // writes the order itself when the top pass is skipped
-            CK(launch_pdl(k_radix_pass<false, false, true>, dim3((unsigned)bn), dim3(kSortThreads), 0, st, 
-                s.ditems_b, s.ditems_a, nullptr, nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu,
-                f.info + kInfoSkipTop, f.order));
-        else
-            CK(launch_pdl(k_radix_pass<false, false>, dim3((unsigned)bn), dim3(kSortThreads), 0, st, 
-                p == 1 ? s.ditems_a : s.ditems_b, p == 1 ? s.ditems_b : s.ditems_a, nullptr, nn, 8 * p, hist,
-                status, s.counters + p, f.info, 0xFFFFFFFFu, nullptr, nullptr));
-        count_launches();
-        CK(cudaGetLastError());
-    }
+    CK(depth_sort_tile(n) == kSortTile ? launch_depth_sort<kSortIpt>(f, s, small_grid, st)
+                                       : launch_depth_sort<kSortIptFew>(f, s, small_grid, st));
     // kept count (k_bin_prep), M and the capacity check (tile-range kernel) are known here
     if (s.walk_chunks > 0) {
         // 3a. two-level counting sort: Gaussians into tile-row lists, then row items into tiles
