@@ -104,13 +104,19 @@ __global__ void __launch_bounds__(1024) k_hist_to_offsets(uint32_t* __restrict__
 // SKIPPABLE (one segment only): when *skip_flag is set, the pass writes only
 // the values, to skip_vals, or, without skip_vals, does nothing (the redundant
 // top pass of a depth sort whose third pass wrote the order).
-template <bool IN_KEYS32, bool OUT_VALS, bool SKIPPABLE = false, int IPT = kSortIpt>
+// COUNTS: digit_base holds the digits' raw counts, and each block forms the offsets.
+// AHEAD (a frame's first pass): the next launch may start before this one ends
+// (k_tiles_small, which needs none of its results and sets the abort flag meanwhile:
+// no block looks at it).
+template <bool IN_KEYS32, bool OUT_VALS, bool SKIPPABLE = false, int IPT = kSortIpt, bool COUNTS = false,
+          bool AHEAD = false>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     const void* __restrict__ in_, void* __restrict__ out_, const uint32_t* __restrict__ d_count, uint32_t count_host,
     int shift, const uint32_t* __restrict__ digit_base, uint32_t* __restrict__ status,
     uint32_t* __restrict__ block_counter, uint32_t* __restrict__ info, uint32_t silent_blk = 0xFFFFFFFFu,
     const uint32_t* __restrict__ skip_flag = nullptr, uint32_t* __restrict__ skip_vals = nullptr) {
     pdl_wait();
+    if (AHEAD) pdl_trigger();
     constexpr int kTile = kSortThreads * IPT;  // items per block
     if (SKIPPABLE && !skip_vals && *skip_flag) return;
     {
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     __shared__ uint32_t s_blk;
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (info && info[kInfoAbort]) return;
+    if (!AHEAD && info && info[kInfoAbort]) return;
     const uint32_t count = d_count ? *d_count : count_host;
     if (tid == 0) s_blk = atomicAdd(block_counter, 1u);
     {
@@ -257,7 +263,9 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
         }
         if (!silent) st_relaxed_u32(&my[tid], kFlagPre | ((excl + cnt) & kValMask));
     }
-    s_delta[tid] = (int32_t)(digit_base[tid] + excl) - (int32_t)local;
+    uint32_t first = digit_base[tid];
+    if (COUNTS) first = block_excl_scan<kSortThreads>(first, s_warp);
+    s_delta[tid] = (int32_t)(first + excl) - (int32_t)local;
     const bool skipped = SKIPPABLE && !OUT_VALS && skip_vals && *skip_flag;  // (read late: fewer live registers)
     __syncthreads();
     // write out: runs of one digit land contiguously; past-the-end items hold the last slots

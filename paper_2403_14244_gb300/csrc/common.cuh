@@ -69,9 +69,12 @@ __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + 
 // while its stream predecessor (a kernel) still runs, and calls pdl_wait()
 // before it touches memory, which returns once the predecessor has finished and
 // its writes are visible. Without the launch attribute pdl_wait() is a no-op.
-// (Kernels do not trigger their successors early: resident waiting CTAs then
-// slowed the predecessors' last waves, measured.)
+// (Kernels do not trigger their successors early, but where a successor has work
+// that needs nothing of them: resident waiting CTAs slowed the predecessors' last
+// waves, measured. Such a successor calls pdl_wait() in one block before it ends,
+// so that what follows it in the stream follows both.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args&&... args) {

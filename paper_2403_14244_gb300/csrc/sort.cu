@@ -313,8 +313,10 @@ __global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(const int32_t* g
 // One block, grid in shared memory (cells <= kGridSmemCells): the row prefix of
 // the difference grid, the tile ranges, the tile-digit histograms, every digit
 // histogram (4 depth + `passes` tile rows) turned into exclusive offsets, and
-// with rowd the row layout of the counting sort (row_layout).
-constexpr int kTilesSmallThreads = 1024;
+// with rowd the row layout of the counting sort (row_layout). 512 threads: their
+// registers fit on an SM beside two blocks of the radix pass that it runs beside.
+constexpr int kTilesSmallThreads = 512;
+constexpr int kTilesSmallDigits = 8 * kRadix / kTilesSmallThreads;  // histogram words per thread
 __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_t* __restrict__ grid, int tiles_x,
                                                                     int tiles_y, int passes, int diff2d,
                                                                     uint2* __restrict__ ranges,
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
                                                                     const int32_t* __restrict__ rowd,
                                                                     uint32_t max_chunks, uint32_t* __restrict__ len,
                                                                     uint32_t* __restrict__ rowinfo) {
-    pdl_wait();
+    // (no wait: it runs beside the depth sort's first pass, which started after the kernel that counted)
     extern __shared__ int32_t s_g[];
     __shared__ uint32_t s_h[8][kRadix];
     __shared__ uint32_t s_warp[kTilesSmallThreads / 32];
@@ -373,9 +375,9 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
     const int rows = 4 + passes;
     __shared__ uint32_t s_wt[8 * kRadix / 32];
     const int lane = tid & 31;
-    uint32_t v[2];
+    uint32_t v[kTilesSmallDigits];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < kTilesSmallDigits; ++r) {
         const int idx = tid + r * kTilesSmallThreads;
         const uint32_t x = idx < rows * kRadix ? (&s_h[0][0])[idx] : 0u;
         uint32_t incl = x;
@@ -389,9 +391,9 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < kTilesSmallDigits; ++r) {
         const int idx = tid + r * kTilesSmallThreads;
-        if (idx < rows * kRadix) {
+        if (idx >= kRadix && idx < rows * kRadix) {  // (the first row stays as counts: the first pass reads it meanwhile)
             uint32_t base = 0;
             for (int k = (idx >> 8) * (kRadix / 32); k < (idx >> 5); ++k) base += s_wt[k];
             hist[idx] = v[r] + base;
@@ -401,6 +403,7 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
         row_layout<kTilesSmallThreads>(rowd, s_g, gx, (uint32_t)tiles_y, (uint32_t)tiles_x,
                                        (uint32_t)min(s_total, (unsigned long long)0xFFFFFFFFu), max_chunks, len,
                                        rowinfo, info, s_warp);
+    pdl_wait();  // ends after the first pass
 }
 
 // ---- counting sort of the entries by tile (route a) ----
@@ -1068,14 +1071,25 @@ SortScratch sort_scratch(const igs_frame& f) {
 // with one silent block (igs_debug_silence_lookback_once).
 std::atomic<int> g_silence_next{0};
 
-// The four passes of a frame's depth sort (small_grid: k_tiles_small decides the top-pass skip).
+// The passes of a frame's depth sort. On a small grid the first one is launched before
+// k_tiles_small, from raw digit counts, and k_tiles_small decides the top-pass skip.
+template <int IPT>
+static cudaError_t launch_first_pass(const igs_frame& f, const SortScratch& s, cudaStream_t st) {
+    const dim3 blocks((unsigned)ceil_div(f.n, kSortThreads * IPT)), threads(kSortThreads);
+    const cudaError_t e = launch_pdl(k_radix_pass<true, false, false, IPT, true, true>, blocks, threads, 0, st,
+                                     f.depth_key, s.ditems_a, nullptr, (uint32_t)f.n, 0, s.hist, s.status_depth,
+                                     s.counters + 0, f.info, g_silence_next.exchange(0) ? 1u : 0xFFFFFFFFu, nullptr,
+                                     nullptr);
+    count_launches();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
 template <int IPT>
 static cudaError_t launch_depth_sort(const igs_frame& f, const SortScratch& s, bool small_grid, cudaStream_t st) {
     const uint32_t nn = (uint32_t)f.n;
     const int64_t bn = ceil_div(f.n, kSortThreads * IPT);
     const dim3 blocks((unsigned)bn), threads(kSortThreads);
     const uint32_t* skip = f.info + kInfoSkipTop;
-    for (int p = 0; p < 4; ++p) {
+    for (int p = small_grid ? 1 : 0; p < 4; ++p) {
         uint32_t* status = s.status_depth + (size_t)p * bn * kRadix;
         const uint32_t* hist = s.hist + p * kRadix;
         cudaError_t e;
@@ -1137,6 +1151,7 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
     const bool walk = s.walk_chunks > 0;
     int32_t* rowd = walk ? s.grid + (size_t)gx * gy : nullptr;  // row differences (route a)
     const uint32_t max2 = walk ? (uint32_t)l2_chunks_max(cap, f.tiles_y) : 0u;
+    const bool few = depth_sort_tile(n) != kSortTile;
     // 0. depth-digit histograms; footprint rows -> per-tile counts -> ranges, tile-digit histograms
     const int prep_blocks = (int)std::min<int64_t>(ceil_div(n, 256), 152 * 4);
     if ((int64_t)gx * gy <= kGridSmemCells)
@@ -1149,12 +1164,16 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
                                                        f.count, nn, gx, gy, s.hist, s.grid, rowd, f.info));
     count_launches();
     CK(cudaGetLastError());
-    if ((int64_t)gx * gy <= kGridSmemCells) {
-        CK(launch_pdl(k_tiles_small, dim3(1), dim3(kTilesSmallThreads), (size_t)gx * gy * 4, st, s.grid, f.tiles_x, f.tiles_y, tp,
-                      footprint == 0 ? 1 : 0,
-                                                                           reinterpret_cast<uint2*>(f.ranges), s.hist,
-                                                                           f.info, (uint64_t)cap, rowd, max2,
-                                                                           s.walk_len, s.walk_rows));
+    const bool small_grid = (int64_t)gx * gy <= kGridSmemCells;
+    if (small_grid) {
+        // the depth sort's first pass, then, beside it, the tile ranges by one block (k_tiles_small was 12 to 16 us of
+        // every frame's chain when it stood before the pass: frames of 200K and of 1M Gaussians 166 and 352 us,
+        // 159 and 342 so)
+        CK(few ? launch_first_pass<kSortIptFew>(f, s, st) : launch_first_pass<kSortIpt>(f, s, st));
+        CK(launch_pdl(k_tiles_small, dim3(1), dim3(kTilesSmallThreads), (size_t)gx * gy * 4, st,
+                      (const int32_t*)s.grid, f.tiles_x, f.tiles_y, tp, footprint == 0 ? 1 : 0,
+                      reinterpret_cast<uint2*>(f.ranges), s.hist, f.info, (uint64_t)cap, (const int32_t*)rowd, max2,
+                      s.walk_len, s.walk_rows));
         count_launches();
         CK(cudaGetLastError());
     } else {
@@ -1171,9 +1190,7 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
         CK(cudaGetLastError());
     }
     // 1. depth sort: (depth_key, index) -> A -> B -> A -> order (or -> order after the third pass)
-    const bool small_grid = (int64_t)gx * gy <= kGridSmemCells;  // k_tiles_small decides the top-pass skip
-    CK(depth_sort_tile(n) == kSortTile ? launch_depth_sort<kSortIpt>(f, s, small_grid, st)
-                                       : launch_depth_sort<kSortIptFew>(f, s, small_grid, st));
+    CK(few ? launch_depth_sort<kSortIptFew>(f, s, small_grid, st) : launch_depth_sort<kSortIpt>(f, s, small_grid, st));
     // kept count (k_bin_prep), M and the capacity check (tile-range kernel) are known here
     if (s.walk_chunks > 0) {
         // 3a. two-level counting sort: Gaussians into tile-row lists, then row items into tiles
