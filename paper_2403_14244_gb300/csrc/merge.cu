@@ -11,15 +11,15 @@
 //                    up together, in index order
 //   k_merge_mark     per sorted position that starts a cell of two or more:
 //                    its members' roles (the first leads, the others go), and
-//                    the position appended to the list of merged cells
-//   k_merge_count    per block of Gaussians: how many are written
+//                    the position of a cell of more than eight in a list
+//   k_merge_count    per block of Gaussians: how many are written, and which
 //   k_merge_scan     one CTA: each block's first output slot, the total
+//   k_merge_cells    a warp per merged cell of more than eight members
 //   k_merge_write    per block of Gaussians: output slots; kept Gaussians copy
-//                    parameters and moments (colour rows cooperatively); a
-//                    leader records its slot for its cell
-//   k_merge_cells    one warp per merged cell: the merged Gaussian (FP32,
-//                    compensated sums over the members in index order, means
-//                    relative to the first member), zero moments
+//                    parameters and moments (colour rows cooperatively); the
+//                    smaller cells led there are merged, eight lanes a cell
+// A merged Gaussian: FP32, compensated sums over the members in index order,
+// means relative to the first member, zero moments.
 //
 // The arithmetic of a merged Gaussian is FP32 (this part's FP64 rate is a small
 // fraction of its FP32 rate): Kahan-compensated sums keep each sum's error at a
@@ -37,8 +37,11 @@ namespace {
 
 constexpr uint32_t kRoleKept = 0xFFFFFFFFu;  // not merged
 constexpr uint32_t kRoleGone = 0xFFFFFFFEu;  // merged into an earlier Gaussian
+constexpr uint32_t kRoleLarge = 0xFFFFFFFDu; // the first of a cell of more than kSmallCell members
+// (any other role: the first of a smaller cell, whose sorted items start there; n < 2^31)
 constexpr int kMergeThreads = 256;
 constexpr int kMergeScanThreads = 1024;
+constexpr int kMergeScanEach = 8;  // block counts per thread and round (one: 20 us at 3M Gaussians, now 11)
 
 struct MergeArrays {
     const float4* ms;
@@ -102,31 +105,47 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_keys(const float4* __re
 
 // Sorted items (key << 32 | index). A position that starts a cell of two or
 // more eligible Gaussians marks its members: role[first] = the start position,
-// role[other members] = gone; and appends the position to `cells`. role is
-// kRoleKept everywhere on entry.
+// or kRoleLarge for more than kSmallCell members, whose start is appended to
+// `cells` (list order is free: each cell's output slot is fixed); role[other
+// members] = gone. role is kRoleKept everywhere on entry.
+constexpr int kSmallCell = 8;
 __global__ void __launch_bounds__(kMergeThreads) k_merge_mark(const u64* __restrict__ items, int64_t n,
                                                               uint32_t* __restrict__ role,
                                                               uint32_t* __restrict__ cells,
                                                               uint32_t* __restrict__ n_cells,
                                                               const uint32_t* __restrict__ info) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n || info[kInfoAbort]) return;  // after a sort that gave up, the items are not a permutation
-    const uint32_t key = (uint32_t)(items[p] >> 32);
-    if (key == 0xFFFFFFFFu) return;
-    if (p > 0 && (uint32_t)(items[p - 1] >> 32) == key) return;  // not the cell's first
-    if (p + 1 >= n || (uint32_t)(items[p + 1] >> 32) != key) return;  // alone in its cell: kept
-    role[(uint32_t)items[p]] = (uint32_t)p;
-    for (int64_t r = p + 1; r < n && (uint32_t)(items[r] >> 32) == key; ++r) role[(uint32_t)items[r]] = kRoleGone;
-    cells[atomicAdd(n_cells, 1u)] = (uint32_t)p;  // (list order is free: each cell's output slot is fixed)
+    if (info[kInfoAbort]) return;  // after a sort that gave up, the items are not a permutation
+    const int lane = threadIdx.x & 31;
+    const u64 it = p < n ? items[p] : ~0ull;
+    const uint32_t key = (uint32_t)(it >> 32);
+    uint32_t prev = __shfl_up_sync(0xffffffffu, key, 1), next = __shfl_down_sync(0xffffffffu, key, 1);
+    if (lane == 0) prev = p > 0 && p < n ? (uint32_t)(items[p - 1] >> 32) : ~key;
+    if (lane == 31) next = p + 1 < n ? (uint32_t)(items[p + 1] >> 32) : ~key;
+    // the cell's first, and not alone in it (past the end the key is that of a Gaussian that is not eligible)
+    if (key == 0xFFFFFFFFu || prev == key || next != key) return;
+    int64_t r = p + 1;
+    for (; r < n; ++r) {
+        const u64 m = items[r];
+        if ((uint32_t)(m >> 32) != key) break;
+        role[(uint32_t)m] = kRoleGone;
+    }
     // (a cell of many Gaussians is marked by one thread: the cost grows with the
     // largest cell, not with n)
+    const bool small = r - p <= kSmallCell;
+    role[(uint32_t)it] = small ? (uint32_t)p : kRoleLarge;
+    if (!small) cells[atomicAdd(n_cells, 1u)] = (uint32_t)p;
 }
 
-// Per block of kMergeThreads Gaussians: the number written (all but the gone).
+// Per block of kMergeThreads Gaussians: the number written (all but the gone), and
+// which, a bit each.
 __global__ void __launch_bounds__(kMergeThreads) k_merge_count(const uint32_t* __restrict__ role, int64_t n,
-                                                               uint32_t* __restrict__ blk) {
+                                                               uint32_t* __restrict__ blk,
+                                                               uint32_t* __restrict__ emit_bits) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool out = i < n && role[i] != kRoleGone;
+    const uint32_t bits = __ballot_sync(0xffffffffu, out);
+    if ((threadIdx.x & 31) == 0) emit_bits[(size_t)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5)] = bits;
     const uint32_t c = __syncthreads_count(out);
     if (threadIdx.x == 0) blk[blockIdx.x] = c;
 }
@@ -144,69 +163,40 @@ __global__ void __launch_bounds__(kMergeScanThreads) k_merge_scan(uint32_t* __re
     __shared__ unsigned long long s_carry;
     if (threadIdx.x == 0) s_carry = 0ull;
     __syncthreads();
-    for (int64_t b0 = 0; b0 < blocks; b0 += kMergeScanThreads) {
-        const int64_t b = b0 + threadIdx.x;
-        const uint32_t v = b < blocks ? blk[b] : 0u;
-        const uint32_t ex = block_excl_scan<kMergeScanThreads>(v, s_warp);
+    for (int64_t b0 = 0; b0 < blocks; b0 += kMergeScanThreads * kMergeScanEach) {
+        const int64_t b = b0 + (int64_t)threadIdx.x * kMergeScanEach;
+        uint32_t v[kMergeScanEach], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kMergeScanEach; ++i) v[i] = b + i < blocks ? blk[b + i] : 0u;
+#pragma unroll
+        for (int i = 0; i < kMergeScanEach; ++i) sum += v[i];
+        const uint32_t ex = block_excl_scan<kMergeScanThreads>(sum, s_warp);
         const unsigned long long carry = s_carry;
-        if (b < blocks) blk[b] = (uint32_t)(carry + ex);
+        uint32_t at = (uint32_t)(carry + ex);
+#pragma unroll
+        for (int i = 0; i < kMergeScanEach; ++i) {
+            if (b + i < blocks) blk[b + i] = at;
+            at += v[i];
+        }
         __syncthreads();
-        if (threadIdx.x == kMergeScanThreads - 1) s_carry = carry + ex + v;
+        if (threadIdx.x == kMergeScanThreads - 1) s_carry = carry + ex + sum;
         __syncthreads();
     }
     if (threadIdx.x == 0) *d_count = (int64_t)s_carry;
 }
 
-// Per block of kMergeThreads Gaussians: output slots by a block scan; kept
-// Gaussians copy their means, scales, opacities and moments (one thread each)
-// and then, cooperatively, their colour rows and moments (float4 when C is a
-// multiple of 4); the leader of a merged cell records its slot at its cell's
-// sorted start position (cell_slot, indexed like the sorted items).
-template <int C>
-__global__ void __launch_bounds__(kMergeThreads) k_merge_write(MergeArrays in, MergeOut out, int64_t n,
-                                                               const uint32_t* __restrict__ role,
-                                                               const uint32_t* __restrict__ blk,
-                                                               uint32_t* __restrict__ cell_slot,
-                                                               const uint32_t* __restrict__ info) {
-    if (info[kInfoAbort]) return;
-    __shared__ uint32_t s_warp[kMergeThreads / 32];
-    __shared__ uint32_t s_dst[kMergeThreads];  // output slot of a kept Gaussian, else ~0
-    const int64_t i0 = (int64_t)blockIdx.x * kMergeThreads, i = i0 + threadIdx.x;
-    const uint32_t rl = i < n ? role[i] : kRoleGone;
-    const bool emit = rl != kRoleGone;
-    const uint32_t slot = blk[blockIdx.x] + block_excl_scan<kMergeThreads>(emit ? 1u : 0u, s_warp);
-    s_dst[threadIdx.x] = rl == kRoleKept ? slot : 0xFFFFFFFFu;
-    const size_t d = slot, s = (size_t)i;
-    if (rl == kRoleKept) {
-        out.ms[d] = in.ms[s];
-        out.m_ms[d] = in.m_ms[s];
-        out.v_ms[d] = in.v_ms[s];
-        out.op[d] = in.op[s];
-        out.m_op[d] = in.m_op[s];
-        out.v_op[d] = in.v_op[s];
-    } else if (emit) {
-        cell_slot[rl] = slot;
-    }
-    __syncthreads();
-    const int nr = (int)min((int64_t)kMergeThreads, n - i0);
-    constexpr int V = (C % 4 == 0) ? 4 : 1;  // floats per access
-    constexpr int CV = C / V;                // accesses per row
-    using T = typename std::conditional<V == 4, float4, float>::type;
-    const T* icol = reinterpret_cast<const T*>(in.col);
-    const T* imc = reinterpret_cast<const T*>(in.m_col);
-    const T* ivc = reinterpret_cast<const T*>(in.v_col);
-    T* ocol = reinterpret_cast<T*>(out.col);
-    T* omc = reinterpret_cast<T*>(out.m_col);
-    T* ovc = reinterpret_cast<T*>(out.v_col);
-    for (int q = threadIdx.x; q < nr * CV; q += kMergeThreads) {
-        const int j = q / CV, f = q - j * CV;
-        const uint32_t dj = s_dst[j];
-        if (dj == 0xFFFFFFFFu) continue;
-        const size_t src = (size_t)(i0 + j) * CV + f, dst = (size_t)dj * CV + f;
-        ocol[dst] = icol[src];
-        omc[dst] = imc[src];
-        ovc[dst] = ivc[src];
-    }
+// Output slot of the cell led by Gaussian i, for eight lanes (sub = 0 .. 7 of a group
+// starting at lane `base`): those written in earlier blocks, and before i in its block.
+__device__ __forceinline__ size_t leader_slot(uint32_t i, int sub, const uint32_t* __restrict__ blk,
+                                              const uint32_t* __restrict__ emit_bits) {
+    static_assert(kMergeThreads == 256, "eight words of bits per block");
+    const uint32_t b = i / kMergeThreads, w = (i % kMergeThreads) / 32;
+    uint32_t bits = emit_bits[(size_t)b * (kMergeThreads / 32) + sub];
+    if ((uint32_t)sub == w) bits &= (1u << (i & 31)) - 1u;
+    uint32_t c = (uint32_t)sub <= w ? (uint32_t)__popc(bits) : 0u;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    return (size_t)blk[b] + c;
 }
 
 // Kahan-compensated sum (s, c): add x.
@@ -222,24 +212,153 @@ __device__ __forceinline__ void kahan_lanes(float& s, float& c, float x, int cnt
     for (int j = 0; j < cnt; ++j) kahan_add(s, c, __shfl_sync(0xffffffffu, x, j));
 }
 
-// One warp per merged cell (a grid-stride loop over the list of cells): lane j
-// holds member j of each run of 32 (index order), and every sum adds the
-// members' terms in index order; colour coefficient c is lane c mod 32's.
+// A member's term of sum o_k (sigma_k^2 + |mu_k - mu|^2 / 3); e = mu - mu_0.
+__device__ __forceinline__ float spread_term(float4 m, float4 m0, float o, float ex, float ey, float ez,
+                                             int param_mode) {
+    const float sk = param_mode == 1 ? expf(m.w) : m.w;
+    const float dx = __fsub_rn(__fsub_rn(m.x, m0.x), ex), dy = __fsub_rn(__fsub_rn(m.y, m0.y), ey),
+                dz = __fsub_rn(__fsub_rn(m.z, m0.z), ez);
+    const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+    return __fmul_rn(o, __fadd_rn(__fmul_rn(sk, sk), __fdiv_rn(d2, 3.0f)));
+}
+
+// A merged Gaussian's parameters but its colour, and their moments (0), into slot d.
+__device__ __forceinline__ void write_merged(MergeOut out, size_t d, float4 m0, float ex, float ey, float ez, float V,
+                                             float W, float L, bool opaque, int param_mode) {
+    const float sigma = sqrtf(__fdiv_rn(V, W));
+    const float cover = opaque ? 1.0f : -expm1f(L);  // 1 - prod (1 - o_k)
+    float o_out;
+    if (param_mode == 1)  // logit: log(cover) - log(1 - cover), or that of 0.99
+        o_out = cover >= 0.99f ? logf(99.0f) : __fsub_rn(logf(cover), L);
+    else
+        o_out = fminf(cover, 0.99f);
+    out.ms[d] = make_float4(__fadd_rn(m0.x, ex), __fadd_rn(m0.y, ey), __fadd_rn(m0.z, ez),
+                            param_mode == 1 ? logf(sigma) : sigma);
+    out.op[d] = o_out;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    out.m_ms[d] = zero;
+    out.v_ms[d] = zero;
+    out.m_op[d] = 0.f;
+    out.v_op[d] = 0.f;
+}
+
+// A merged cell of at most kSmallCell members (sorted items from p0 on, output slot d;
+// have: there is one) per eight lanes, four to a warp: lane j of the eight holds its
+// member j, and every sum adds the members' terms in index order, as k_merge_cells
+// does; a colour row is read and written by the eight lanes together.
+template <int C>
+__device__ __forceinline__ void merge_small(const MergeArrays& in, const MergeOut& out, int64_t n, int param_mode,
+                                            const u64* __restrict__ items, int64_t p0, size_t d, bool have) {
+    constexpr int V = (C % 4 == 0) ? 4 : 1;  // floats per access
+    constexpr int CV = C / V;                // accesses per row
+    constexpr int CL = (CV + kSmallCell - 1) / kSmallCell;  // accesses per lane
+    using T = typename std::conditional<V == 4, float4, float>::type;
+    constexpr uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sub = lane & (kSmallCell - 1), base = lane - sub;
+    const int64_t r = p0 + sub;
+    const u64 it = have && r < n ? items[r] : 0ull;
+    const uint32_t key = __shfl_sync(kAll, (uint32_t)(it >> 32), base);
+    const bool mem = have && r < n && (uint32_t)(it >> 32) == key;
+    const uint32_t ball = (__ballot_sync(kAll, mem) >> base) & ((1u << kSmallCell) - 1u);
+    const int cnt = __popc(ball);  // (sorted: the members are the first cnt lanes)
+    const uint32_t k = (uint32_t)it;
+    float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+    float o = 0.f, lk = 0.f;
+    if (mem) {
+        m = in.ms[k];
+        opacity_terms(in.op[k], param_mode, o, lk);
+    }
+    const float4 m0 = make_float4(__shfl_sync(kAll, m.x, base), __shfl_sync(kAll, m.y, base),
+                                  __shfl_sync(kAll, m.z, base), 0.f);
+    const float x = __fmul_rn(o, __fsub_rn(m.x, m0.x)), y = __fmul_rn(o, __fsub_rn(m.y, m0.y)),
+                z = __fmul_rn(o, __fsub_rn(m.z, m0.z));
+    const bool opaque = ((__ballot_sync(kAll, mem && isinf(lk)) >> base) & ((1u << kSmallCell) - 1u)) != 0;
+    if (isinf(lk)) lk = 0.f;
+    const int most = __reduce_max_sync(kAll, cnt);  // of the warp's cells
+    float W = 0.f, cW = 0.f, ox = 0.f, cx = 0.f, oy = 0.f, cy = 0.f, oz = 0.f, cz = 0.f, L = 0.f, cL = 0.f;
+    for (int j = 0; j < most; ++j) {
+        const float oj = __shfl_sync(kAll, o, base + j), xj = __shfl_sync(kAll, x, base + j),
+                    yj = __shfl_sync(kAll, y, base + j), zj = __shfl_sync(kAll, z, base + j),
+                    lj = __shfl_sync(kAll, lk, base + j);
+        if (j < cnt) {
+            kahan_add(W, cW, oj);
+            kahan_add(ox, cx, xj);
+            kahan_add(oy, cy, yj);
+            kahan_add(oz, cz, zj);
+            kahan_add(L, cL, lj);
+        }
+    }
+    const float ex = __fdiv_rn(ox, W), ey = __fdiv_rn(oy, W), ez = __fdiv_rn(oz, W);  // mean - mu_0
+    const float t = mem ? spread_term(m, m0, o, ex, ey, ez, param_mode) : 0.f;
+    float Vs = 0.f, cV = 0.f, acc[CL * V], comp[CL * V];
+#pragma unroll
+    for (int q = 0; q < CL * V; ++q) acc[q] = comp[q] = 0.f;
+    for (int j0 = 0; j0 < most; j0 += 2) {  // the rows of two members read together
+        T row[2][CL];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const uint32_t kj = __shfl_sync(kAll, k, base + ((j0 + u) & (kSmallCell - 1)));
+            const T* src = reinterpret_cast<const T*>(in.col) + (size_t)kj * CV;
+#pragma unroll
+            for (int q = 0; q < CL; ++q) {
+                row[u][q] = T{};
+                if (j0 + u < cnt && sub + kSmallCell * q < CV) row[u][q] = src[sub + kSmallCell * q];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = (j0 + u) & (kSmallCell - 1);
+            const float oj = __shfl_sync(kAll, o, base + j), tj = __shfl_sync(kAll, t, base + j);
+            if (j0 + u < cnt) {
+                kahan_add(Vs, cV, tj);
+#pragma unroll
+                for (int q = 0; q < CL; ++q)
+#pragma unroll
+                    for (int f = 0; f < V; ++f)
+                        kahan_add(acc[q * V + f], comp[q * V + f],
+                                  __fmul_rn(oj, reinterpret_cast<const float*>(&row[u][q])[f]));
+            }
+        }
+    }
+    if (!have) return;  // (no warp-wide step below)
+    if (sub == 0) write_merged(out, d, m0, ex, ey, ez, Vs, W, L, opaque, param_mode);
+    T* oc = reinterpret_cast<T*>(out.col) + d * CV;
+    T* om = reinterpret_cast<T*>(out.m_col) + d * CV;
+    T* ov = reinterpret_cast<T*>(out.v_col) + d * CV;
+#pragma unroll
+    for (int q = 0; q < CL; ++q) {
+        const int c = sub + kSmallCell * q;
+        if (c < CV) {
+            T v;
+#pragma unroll
+            for (int f = 0; f < V; ++f) reinterpret_cast<float*>(&v)[f] = __fdiv_rn(acc[q * V + f], W);
+            oc[c] = v;
+            om[c] = T{};
+            ov[c] = T{};
+        }
+    }
+}
+
+// Merged cells of more than kSmallCell members, one to a warp (a grid-stride loop over
+// the list): lane j holds member j of each run of 32 (index order), and every sum adds
+// the members' terms in index order; colour coefficient c is lane c mod 32's.
 template <int C>
 __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, MergeOut out, int64_t n,
                                                                int param_mode, const u64* __restrict__ items,
                                                                const uint32_t* __restrict__ cells,
                                                                const uint32_t* __restrict__ n_cells,
-                                                               const uint32_t* __restrict__ cell_slot,
+                                                               const uint32_t* __restrict__ blk,
+                                                               const uint32_t* __restrict__ emit_bits,
                                                                const uint32_t* __restrict__ info) {
+    pdl_trigger();  // k_merge_write needs nothing written here
     if (info[kInfoAbort]) return;
-    const int lane = threadIdx.x & 31;
     const uint32_t total = *n_cells;
+    const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (kMergeThreads / 32);
     for (uint32_t g = blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5); g < total; g += warps) {
         const int64_t p0 = cells[g];
         const uint32_t key = (uint32_t)(items[p0] >> 32);
-        const size_t d = cell_slot[p0];
+        const size_t d = leader_slot((uint32_t)items[p0], lane & 7, blk, emit_bits);
         const float4 m0 = in.ms[(uint32_t)items[p0]];  // the first member: origin of the offsets
         // W = sum o_k, offsets sum o_k (mu_k - mu_0), L = sum log(1 - o_k) over the members
         float W = 0.f, cW = 0.f, ox = 0.f, cx = 0.f, oy = 0.f, cy = 0.f, oz = 0.f, cz = 0.f, L = 0.f, cL = 0.f;
@@ -295,31 +414,11 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, M
                     float lk;
                     opacity_terms(in.op[k], param_mode, o, lk);
                 }
-                const float sk = param_mode == 1 ? expf(m.w) : m.w;
-                const float dx = __fsub_rn(__fsub_rn(m.x, m0.x), ex), dy = __fsub_rn(__fsub_rn(m.y, m0.y), ey),
-                            dz = __fsub_rn(__fsub_rn(m.z, m0.z), ez);
-                const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-                t = __fmul_rn(o, __fadd_rn(__fmul_rn(sk, sk), __fdiv_rn(d2, 3.0f)));
+                t = spread_term(m, m0, o, ex, ey, ez, param_mode);
             }
             kahan_lanes(V, cV, t, cnt);
         }
-        if (lane == 0) {
-            const float sigma = sqrtf(__fdiv_rn(V, W));
-            const float cover = opaque ? 1.0f : -expm1f(L);  // 1 - prod (1 - o_k)
-            float o_out;
-            if (param_mode == 1)  // logit: log(cover) - log(1 - cover), or that of 0.99
-                o_out = cover >= 0.99f ? logf(99.0f) : __fsub_rn(logf(cover), L);
-            else
-                o_out = fminf(cover, 0.99f);
-            out.ms[d] = make_float4(__fadd_rn(m0.x, ex), __fadd_rn(m0.y, ey), __fadd_rn(m0.z, ez),
-                                    param_mode == 1 ? logf(sigma) : sigma);
-            out.op[d] = o_out;
-            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-            out.m_ms[d] = zero;
-            out.v_ms[d] = zero;
-            out.m_op[d] = 0.f;
-            out.v_op[d] = 0.f;
-        }
+        if (lane == 0) write_merged(out, d, m0, ex, ey, ez, V, W, L, opaque, param_mode);
         // colour: coefficients lane, lane + 32, ...: sum o_k c_k / W
         constexpr int CP = (C + 31) / 32;  // coefficients per lane
         float acc[CP], cacc[CP];
@@ -368,10 +467,99 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, M
     }
 }
 
+// Per block of kMergeThreads Gaussians: output slots by a block scan; kept
+// Gaussians copy their means, scales, opacities and moments (one thread each)
+// and then, cooperatively, their colour rows and moments (float4 when C is a
+// multiple of 4); and the small cells that a Gaussian of the block leads are
+// merged, eight lanes a cell. Bound by memory bandwidth (3M Gaussians, degree 3:
+// 3.2 GB). A cell's work is a chain of dependent reads; done here, those of some
+// blocks run under the copies of others: 555 us, where the copies took 489 and, after
+// them, a warp per cell 330 (158 as four cells to a warp; as a kernel beside this one
+// no less in all: its reads then wait on the copies'). Four blocks per SM and four
+// accesses in flight: with two 23 us more, five blocks 37, three 43.
+// Runs beside k_merge_cells, whose launch it follows without waiting for it. Its last
+// block ends after k_merge_cells, so that what follows in the stream finds both.
+template <int C>
+__global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in, MergeOut out, int64_t n, int param_mode,
+                                                               const u64* __restrict__ items,
+                                                               const uint32_t* __restrict__ role,
+                                                               const uint32_t* __restrict__ blk,
+                                                               const uint32_t* __restrict__ info) {
+    if (info[kInfoAbort]) {
+        if (blockIdx.x == gridDim.x - 1) pdl_wait();
+        return;
+    }
+    __shared__ uint32_t s_warp[kMergeThreads / 32];
+    __shared__ uint32_t s_dst[kMergeThreads];  // output slot of a kept Gaussian, else ~0
+    __shared__ uint2 s_lead[kMergeThreads];    // small cells led here: start of the items, output slot
+    __shared__ uint32_t s_leads;
+    const int64_t i0 = (int64_t)blockIdx.x * kMergeThreads, i = i0 + threadIdx.x;
+    const uint32_t rl = i < n ? role[i] : kRoleGone;
+    if (threadIdx.x == 0) s_leads = 0u;
+    const uint32_t slot = blk[blockIdx.x] + block_excl_scan<kMergeThreads>(rl != kRoleGone ? 1u : 0u, s_warp);
+    s_dst[threadIdx.x] = rl == kRoleKept ? slot : 0xFFFFFFFFu;
+    const size_t d = slot, s = (size_t)i;
+    if (rl == kRoleKept) {
+        out.ms[d] = in.ms[s];
+        out.m_ms[d] = in.m_ms[s];
+        out.v_ms[d] = in.v_ms[s];
+        out.op[d] = in.op[s];
+        out.m_op[d] = in.m_op[s];
+        out.v_op[d] = in.v_op[s];
+    } else if (rl < kRoleLarge) {
+        s_lead[atomicAdd(&s_leads, 1u)] = make_uint2(rl, slot);
+    }
+    __syncthreads();
+    const int nr = (int)min((int64_t)kMergeThreads, n - i0);
+    constexpr int V = (C % 4 == 0) ? 4 : 1;  // floats per access
+    constexpr int CV = C / V;                // accesses per row
+    using T = typename std::conditional<V == 4, float4, float>::type;
+    const T* icol = reinterpret_cast<const T*>(in.col);
+    const T* imc = reinterpret_cast<const T*>(in.m_col);
+    const T* ivc = reinterpret_cast<const T*>(in.v_col);
+    T* ocol = reinterpret_cast<T*>(out.col);
+    T* omc = reinterpret_cast<T*>(out.m_col);
+    T* ovc = reinterpret_cast<T*>(out.v_col);
+    constexpr int U = 4;  // accesses of each array in flight per thread
+    for (int q0 = threadIdx.x; q0 < nr * CV; q0 += U * kMergeThreads) {
+        T a[U], b[U], c[U];
+        size_t dst[U];
+        bool on[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * kMergeThreads, j = q / CV, f = q - j * CV;
+            const uint32_t dj = q < nr * CV ? s_dst[j] : 0xFFFFFFFFu;
+            on[u] = dj != 0xFFFFFFFFu;
+            dst[u] = (size_t)dj * CV + f;
+            if (on[u]) {
+                const size_t src = (size_t)(i0 + j) * CV + f;
+                a[u] = icol[src];
+                b[u] = imc[src];
+                c[u] = ivc[src];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (on[u]) {
+                ocol[dst[u]] = a[u];
+                omc[dst[u]] = b[u];
+                ovc[dst[u]] = c[u];
+            }
+    }
+    const uint32_t leads = s_leads;
+    for (uint32_t l0 = (threadIdx.x & ~31) / kSmallCell; l0 < leads; l0 += kMergeThreads / kSmallCell) {
+        const uint32_t l = l0 + (threadIdx.x & 31) / kSmallCell;
+        const uint2 c = l < leads ? s_lead[l] : make_uint2(0u, 0u);
+        merge_small<C>(in, out, n, param_mode, items, c.x, c.y, l < leads);
+        __syncwarp();
+    }
+    if (blockIdx.x == gridDim.x - 1) pdl_wait();
+}
+
 // Work layout (all 256-byte aligned pieces).
 struct MergeWork {
-    uint32_t* key;      // [n] cell keys; after the sort, the output slot of each merged cell (by sorted start)
-    uint32_t* cells;    // [n] sorted start positions of the merged cells
+    uint32_t* key;      // [n] cell keys; after the sort, a bit per Gaussian (emit_bits)
+    uint32_t* cells;    // [n] sorted start positions of the large merged cells
     u64* items_a;       // [n]
     u64* items_b;       // [n]
     uint32_t* role;     // [n]
@@ -436,17 +624,14 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
     k_hist<<<(unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 4), 256, 0, st>>>(w.key, nn, 4, w.hist);
     count_launches();
     CK(cudaGetLastError());
-    k_hist_to_offsets<<<1, 1024, 0, st>>>(w.hist, 4);
-    count_launches();
-    CK(cudaGetLastError());
     for (int p = 0; p < 4; ++p) {  // (key, index) -> A -> B -> A -> B
         uint32_t* status = w.status + (size_t)p * sb * kRadix;
         const uint32_t* hist = w.hist + p * kRadix;
         if (p == 0)
-            k_radix_pass<true, false><<<(unsigned)sb, kSortThreads, 0, st>>>(w.key, w.items_a, nullptr, nn, 0, hist,
+            k_radix_pass<true, false, false, kSortIpt, true><<<(unsigned)sb, kSortThreads, 0, st>>>(w.key, w.items_a, nullptr, nn, 0, hist,
                                                                              status, w.counters + p, w.info);
         else
-            k_radix_pass<false, false><<<(unsigned)sb, kSortThreads, 0, st>>>(
+            k_radix_pass<false, false, false, kSortIpt, true><<<(unsigned)sb, kSortThreads, 0, st>>>(
                 p % 2 ? w.items_a : w.items_b, p % 2 ? w.items_b : w.items_a, nullptr, nn, 8 * p, hist, status,
                 w.counters + p, w.info);
         count_launches();
@@ -456,7 +641,8 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
     k_merge_mark<<<(unsigned)blocks, kMergeThreads, 0, st>>>(sorted, n, w.role, w.cells, w.counters + 8, w.info);
     count_launches();
     CK(cudaGetLastError());
-    k_merge_count<<<(unsigned)blocks, kMergeThreads, 0, st>>>(w.role, n, w.blk);
+    uint32_t* emit_bits = w.key;  // the keys are not read after the first radix pass
+    k_merge_count<<<(unsigned)blocks, kMergeThreads, 0, st>>>(w.role, n, w.blk, emit_bits);
     count_launches();
     CK(cudaGetLastError());
     k_merge_scan<<<1, kMergeScanThreads, 0, st>>>(w.blk, blocks, d_count, w.info);
@@ -466,16 +652,18 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
                    in_m[1], in_m[2], reinterpret_cast<const float4*>(in_v[0]), in_v[1], in_v[2]};
     MergeOut out{reinterpret_cast<float4*>(out_p[0]), out_p[1], out_p[2], reinterpret_cast<float4*>(out_m[0]),
                  out_m[1], out_m[2], reinterpret_cast<float4*>(out_v[0]), out_v[1], out_v[2]};
-    uint32_t* cell_slot = w.key;  // the keys are not read after the first radix pass
-    const unsigned cell_blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 16), 152 * 8));
+    // at most two blocks per SM (half its registers): k_merge_write runs in what is left
+    const unsigned cell_blocks =
+        (unsigned)std::min<int64_t>(ceil_div(n, (kSmallCell + 1) * kMergeThreads / 32), 152 * 2);
     switch (C) {  // colour floats per Gaussian: a compile-time row length for the cooperative copies
 #define IGS_MERGE_C(CC)                                                                                             \
     case CC:                                                                                                        \
-        k_merge_write<CC><<<(unsigned)blocks, kMergeThreads, 0, st>>>(in, out, n, w.role, w.blk, cell_slot, w.info); \
+        k_merge_cells<CC><<<cell_blocks, kMergeThreads, 0, st>>>(in, out, n, param_mode, sorted, w.cells,            \
+                                                                 w.counters + 8, w.blk, emit_bits, w.info);         \
         count_launches();                                                                                           \
         CK(cudaGetLastError());                                                                                     \
-        k_merge_cells<CC><<<cell_blocks, kMergeThreads, 0, st>>>(in, out, n, param_mode, sorted, w.cells,            \
-                                                                 w.counters + 8, cell_slot, w.info);                \
+        CK(launch_pdl(k_merge_write<CC>, dim3((unsigned)blocks), dim3(kMergeThreads), 0, st, in, out, n, param_mode, \
+                      sorted, (const uint32_t*)w.role, (const uint32_t*)w.blk, (const uint32_t*)w.info));           \
         count_launches();                                                                                           \
         CK(cudaGetLastError());                                                                                     \
         break;
