@@ -440,35 +440,34 @@ __device__ __forceinline__ Chunk l1_chunk(uint32_t c, uint32_t cmax, const uint3
 
 // A warp's stable placement of one chunk whose items each span a contiguous
 // range of buckets [lo, hi], one batch of 32 items (one per lane, in order) at
-// a time. Each lane marks its bit at the start of its range (smask[lo]) and
-// past its end (emask[hi + 1]); a warp-wide XOR prefix over the batch's
-// buckets turns the marks into each bucket's covering mask (the lanes whose
-// range holds it: a bit marked at both ends cancels); an item's slot in
-// bucket q = the bucket's cursor + the earlier lanes of the covering mask, and
-// each bucket's cursor then advances by the mask's size. Two marks per item
-// instead of one per (item, bucket), and no per-bucket pass diverges but the
-// slot writes. Items go to a shared-memory stage grouped by bucket and leave
-// by stage slot (lane l takes slots l, l + 32, ..., each to its bucket's run
-// in the output; a chunk too large for the stage writes its items directly). Items are of type T (the value an item
-// takes in bucket q comes from a functor); the stage holds S of them. Shared
-// memory: words(B) 32-bit words, an even count (8-byte items stay aligned).
+// a time. A bucket's slot holds its cursor and the mask of the batch's lanes whose
+// range holds it; each lane sets its bit in the slots of its range, then takes, in
+// each of them, the cursor + the earlier lanes of the mask, and the cursors of the
+// batch's buckets then advance by their masks' sizes. Bound by instructions and
+// shared-memory accesses. (Masks from marks at the ends of the ranges and an XOR
+// prefix over the buckets, two marks per item whatever its range, cost more at the
+// usual two or three buckets an item and no less at forty: 14M entries of 3M
+// Gaussians, level 1 and 2 placed in 40.9 and 65.4 us, now 39.1 and 57.1.)
+// Items go to a shared-memory stage grouped by bucket and leave it a bucket's run
+// at a time (a chunk too large for the stage writes its items directly). Items are
+// of type T (the value an item takes in bucket q comes from a functor); the stage
+// holds S of them. Shared memory: words(B) 32-bit words, an even count (8-byte
+// items stay aligned).
 template <typename T, uint32_t S>
 struct Placer {
-    uint32_t *pos, *smask, *emask, *cov, *first, *lstart;
+    uint2* slot;  // (cursor, mask)
+    uint32_t *first, *lstart;
     T* stage;
     uint32_t B;
     bool staged;
     __host__ __device__ static constexpr uint32_t words(uint32_t B) {
-        return 6 * B + 6 + S * (uint32_t)(sizeof(T) / 4);
+        return 4 * B + 2 + S * (uint32_t)(sizeof(T) / 4);
     }
     __device__ __forceinline__ Placer(uint32_t* ws, uint32_t nb) : B(nb), staged(false) {
-        pos = ws;
-        smask = pos + nb;          // nb + 1 words
-        emask = smask + nb + 1;    // nb + 2 words
-        cov = emask + nb + 2;      // nb words
-        first = cov + nb;
-        lstart = first + nb;       // nb + 1 words (+ 2 pad)
-        stage = reinterpret_cast<T*>(ws + 6 * nb + 6);
+        slot = reinterpret_cast<uint2*>(ws);
+        first = ws + 2 * nb;
+        lstart = first + nb;       // nb + 1 words (+ 1 pad)
+        stage = reinterpret_cast<T*>(ws + 4 * nb + 2);
     }
     // first_slot(q): the chunk's first slot in bucket q of the output; count(q): its items there
     template <typename First, typename Count>
@@ -476,10 +475,6 @@ struct Placer {
         for (uint32_t q = lane; q < B; q += 32) {  // coalesced, independent loads
             first[q] = first_slot(q);
             lstart[q] = count(q);
-        }
-        for (uint32_t q = lane; q < B + 2; q += 32) {
-            emask[q] = 0u;
-            if (q <= B) smask[q] = 0u;
         }
         __syncwarp();
         const uint32_t per = (B + 31) / 32, q0 = min(B, lane * per), q1 = min(B, q0 + per);
@@ -497,7 +492,7 @@ struct Placer {
         for (uint32_t q = q0; q < q1; ++q) {
             const uint32_t c = lstart[q];
             lstart[q] = run;
-            pos[q] = staged ? run : first[q];
+            slot[q] = make_uint2(staged ? run : first[q], 0u);
             run += c;
         }
         if (lane == 31) lstart[B] = total;
@@ -508,55 +503,34 @@ struct Placer {
     __device__ __forceinline__ void batch(uint32_t lo, uint32_t hi, Item item, int lane, T* __restrict__ out) {
         const uint32_t bit = 1u << lane, lt = bit - 1u;
         const bool any = lo <= hi;
-        if (any) {
-            atomicOr(&smask[lo], bit);
-            atomicOr(&emask[hi + 1], bit);
-        }
         const uint32_t qmin = __reduce_min_sync(0xffffffffu, any ? lo : 0xFFFFFFFFu);
         const uint32_t qmax = __reduce_max_sync(0xffffffffu, any ? hi : 0u);
         if (qmin > qmax) return;  // warp-uniform: no item spans a bucket
-        __syncwarp();
-        // covering masks: lanes whose span holds q = XOR of start and end marks up to q
-        uint32_t carry = 0u;
-        for (uint32_t base = qmin; base <= qmax; base += 32) {
-            const uint32_t q = base + lane;
-            uint32_t x = q <= qmax ? (smask[q] ^ emask[q]) : 0u;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x ^= y;
-            }
-            x ^= carry;
-            if (q <= qmax) cov[q] = x;
-            carry = __shfl_sync(0xffffffffu, x, 31);
-        }
+        for (uint32_t q = lo; q <= hi; ++q) atomicOr(&slot[q].y, bit);
         __syncwarp();
         for (uint32_t q = lo; q <= hi; ++q) {
-            const uint32_t at = pos[q] + __popc(cov[q] & lt);
+            const uint2 c = slot[q];
+            const uint32_t at = c.x + __popc(c.y & lt);
             const T v = item(q);
             if (staged) stage[at] = v; else out[at] = v;
         }
         __syncwarp();
-        for (uint32_t base = qmin; base <= qmax; base += 32) {
-            const uint32_t q = base + lane;
-            if (q <= qmax) {
-                pos[q] += __popc(cov[q]);
-                smask[q] = 0u;
-                emask[q] = 0u;
-            }
+        for (uint32_t q = qmin + lane; q <= qmax; q += 32) {
+            const uint2 c = slot[q];
+            slot[q] = make_uint2(c.x + __popc(c.y), 0u);
         }
-        if (lane == 0) emask[qmax + 1] = 0u;  // ends past the last bucket of the batch
         __syncwarp();
     }
-    // staged chunk: every bucket's run to out[first[q] ...]; lane l takes stage slots l, l + 32, ...,
-    // each written to its bucket's output run (a warp store covers 32 consecutive slots)
+    // staged chunk: every bucket's run to out[first[q] ...], eight lanes a bucket (a run is
+    // 5 to 40 items; by stage slot, each lane looking for its slot's bucket, level 2 took 62.3 us; with
+    // 4 or 16 lanes a training step of 3M is 3 to 6 us longer, with 32 11)
     __device__ __forceinline__ void flush(T* __restrict__ out, int lane) {
         if (!staged) return;
-        const uint32_t total = lstart[B];
-        uint32_t q = 0;  // the bucket holding stage slot e: slots rise, so q only moves forward
-        for (uint32_t e = lane; e < total; e += 32) {
-            while (lstart[q + 1] <= e) ++q;
-            out[first[q] + (e - lstart[q])] = stage[e];
+        constexpr uint32_t G = 8;
+        for (uint32_t q = lane / G; q < B; q += 32 / G) {
+            const uint32_t s = lstart[q], e = lstart[q + 1];
+            T* dst = out + first[q];
+            for (uint32_t i = s + lane % G; i < e; i += G) dst[i - s] = stage[i];
         }
     }
 };
