@@ -4,11 +4,13 @@
 // share a cell of a grid, two or more of them, become one Gaussian at the
 // place of the first; every other Gaussian is kept. Output in index order.
 //
-//   k_merge_keys     per Gaussian: its cell key (x | y << 10 | z << 20) if it
-//                    is eligible, else 0xFFFFFFFF (FP32 cell indices, each step
-//                    rounded once; the opacity floor tested on the stored value)
-//   k_hist, 4 passes stable radix sort of (key, index): a cell's Gaussians end
-//                    up together, in index order
+//   k_merge_keys     per Gaussian: its cell key (the bits of x, y, z
+//                    interleaved) if it is eligible, else 0xFFFFFFFF (FP32 cell
+//                    indices, each step rounded once; the opacity floor tested
+//                    on the stored value); the keys' digit counts
+//   4 passes         stable radix sort of (key, index): a cell's Gaussians end
+//                    up together, in index order; the fourth returns at once
+//                    when the keys fit three
 //   k_merge_mark     per sorted position that starts a cell of two or more:
 //                    its members' roles (the first leads, the others go), and
 //                    the position of a cell of more than eight in a list
@@ -85,23 +87,72 @@ __device__ __forceinline__ void opacity_terms(float x, int param_mode, float& o,
     }
 }
 
+// Bit i of a 10-bit number to bit 3 i.
+__device__ __forceinline__ uint32_t spread3(uint32_t x) {
+    x = (x | (x << 16)) & 0x030000FFu;
+    x = (x | (x << 8)) & 0x0300F00Fu;
+    x = (x | (x << 4)) & 0x030C30C3u;
+    return (x | (x << 2)) & 0x09249249u;
+}
+
+// Interleaved, the keys of cells below 256 in every axis are below 2^24: three passes
+// then sort them, unless a key is 2^24 - 1, whose digits an ineligible Gaussian shares.
+// *three (not zero on entry) is cleared by a key that needs the fourth. hist [4][256]:
+// the digits' counts (zero on entry); those that most of a warp shares, of ineligible
+// Gaussians and of a top byte 0, are added once per warp. (3M Gaussians: keys of three
+// 10-bit fields, their digits counted by a kernel of its own, took 34 us and four passes
+// of 24; now 28 and three: the merge 748 -> 725 us.)
 __global__ void __launch_bounds__(kMergeThreads) k_merge_keys(const float4* __restrict__ ms,
                                                               const float* __restrict__ op, int64_t n,
                                                               int param_mode, float lox, float loy, float loz,
-                                                              float inv, float scale_max, uint32_t* __restrict__ key) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4 m = ms[i];
-    uint32_t k = 0xFFFFFFFFu;
-    if (isfinite(m.x) && isfinite(m.y) && isfinite(m.z) && m.w <= scale_max && opacity_eligible(op[i], param_mode)) {
-        const float cx = floorf(__fmul_rn(__fsub_rn(m.x, lox), inv));
-        const float cy = floorf(__fmul_rn(__fsub_rn(m.y, loy), inv));
-        const float cz = floorf(__fmul_rn(__fsub_rn(m.z, loz), inv));
-        if (cx >= 0.f && cx < 1024.f && cy >= 0.f && cy < 1024.f && cz >= 0.f && cz < 1024.f)
-            k = (uint32_t)cx | ((uint32_t)cy << 10) | ((uint32_t)cz << 20);
+                                                              float inv, float scale_max, uint32_t* __restrict__ key,
+                                                              uint32_t* __restrict__ hist,
+                                                              uint32_t* __restrict__ three) {
+    __shared__ uint32_t s_h[4][kRadix];
+    for (int q = threadIdx.x; q < 4 * kRadix; q += kMergeThreads) (&s_h[0][0])[q] = 0u;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    bool wide = false;
+    for (int64_t i0 = (int64_t)blockIdx.x * kMergeThreads; i0 < n; i0 += (int64_t)gridDim.x * kMergeThreads) {
+        const int64_t i = i0 + threadIdx.x;
+        uint32_t k = 0xFFFFFFFFu;
+        if (i < n) {
+            const float4 m = ms[i];
+            if (isfinite(m.x) && isfinite(m.y) && isfinite(m.z) && m.w <= scale_max &&
+                opacity_eligible(op[i], param_mode)) {
+                const float cx = floorf(__fmul_rn(__fsub_rn(m.x, lox), inv));
+                const float cy = floorf(__fmul_rn(__fsub_rn(m.y, loy), inv));
+                const float cz = floorf(__fmul_rn(__fsub_rn(m.z, loz), inv));
+                if (cx >= 0.f && cx < 1024.f && cy >= 0.f && cy < 1024.f && cz >= 0.f && cz < 1024.f)
+                    k = spread3((uint32_t)cx) | (spread3((uint32_t)cy) << 1) | (spread3((uint32_t)cz) << 2);
+            }
+            key[i] = k;
+        }
+        const bool out = i < n && k == 0xFFFFFFFFu, in = i < n && !out;
+        wide |= in && k >= 0x00FFFFFFu;
+        const uint32_t outs = __popc(__ballot_sync(0xffffffffu, out));
+        const uint32_t zeros = __popc(__ballot_sync(0xffffffffu, in && (k >> 24) == 0u));
+        if (lane < 4 && outs) atomicAdd(&s_h[lane][kRadix - 1], outs);
+        if (lane == 0 && zeros) atomicAdd(&s_h[3][0], zeros);
+        if (in) {
+#pragma unroll
+            for (int p = 0; p < 3; ++p) atomicAdd(&s_h[p][(k >> (8 * p)) & 0xFFu], 1u);
+            if (k >> 24) atomicAdd(&s_h[3][k >> 24], 1u);
+        }
     }
-    key[i] = k;
+    if (__syncthreads_or(wide) && threadIdx.x == 0) *three = 0u;  // (every writer writes the same)
+    for (int q = threadIdx.x; q < 4 * kRadix; q += kMergeThreads) {
+        const uint32_t c = (&s_h[0][0])[q];
+        if (c) atomicAdd(&hist[q], c);
+    }
 }
+
+// The sorted (key << 32 | index): after three passes in one buffer, after four in the other.
+struct SortedItems {
+    const u64 *three_passes, *four_passes;
+    const uint32_t* three;
+    __device__ __forceinline__ const u64* get() const { return *three ? three_passes : four_passes; }
+};
 
 // Sorted items (key << 32 | index). A position that starts a cell of two or
 // more eligible Gaussians marks its members: role[first] = the start position,
@@ -109,11 +160,12 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_keys(const float4* __re
 // `cells` (list order is free: each cell's output slot is fixed); role[other
 // members] = gone. role is kRoleKept everywhere on entry.
 constexpr int kSmallCell = 8;
-__global__ void __launch_bounds__(kMergeThreads) k_merge_mark(const u64* __restrict__ items, int64_t n,
+__global__ void __launch_bounds__(kMergeThreads) k_merge_mark(SortedItems sorted, int64_t n,
                                                               uint32_t* __restrict__ role,
                                                               uint32_t* __restrict__ cells,
                                                               uint32_t* __restrict__ n_cells,
                                                               const uint32_t* __restrict__ info) {
+    const u64* __restrict__ items = sorted.get();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (info[kInfoAbort]) return;  // after a sort that gave up, the items are not a permutation
     const int lane = threadIdx.x & 31;
@@ -344,7 +396,7 @@ __device__ __forceinline__ void merge_small(const MergeArrays& in, const MergeOu
 // the members' terms in index order; colour coefficient c is lane c mod 32's.
 template <int C>
 __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, MergeOut out, int64_t n,
-                                                               int param_mode, const u64* __restrict__ items,
+                                                               int param_mode, SortedItems sorted,
                                                                const uint32_t* __restrict__ cells,
                                                                const uint32_t* __restrict__ n_cells,
                                                                const uint32_t* __restrict__ blk,
@@ -353,6 +405,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, M
     pdl_trigger();  // k_merge_write needs nothing written here
     if (info[kInfoAbort]) return;
     const uint32_t total = *n_cells;
+    const u64* __restrict__ items = sorted.get();
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (kMergeThreads / 32);
     for (uint32_t g = blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5); g < total; g += warps) {
@@ -481,8 +534,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, M
 // block ends after k_merge_cells, so that what follows in the stream finds both.
 template <int C>
 __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in, MergeOut out, int64_t n, int param_mode,
-                                                               const u64* __restrict__ items,
-                                                               const uint32_t* __restrict__ role,
+                                                               SortedItems sorted, const uint32_t* __restrict__ role,
                                                                const uint32_t* __restrict__ blk,
                                                                const uint32_t* __restrict__ info) {
     if (info[kInfoAbort]) {
@@ -547,6 +599,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in
             }
     }
     const uint32_t leads = s_leads;
+    const u64* __restrict__ items = sorted.get();
     for (uint32_t l0 = (threadIdx.x & ~31) / kSmallCell; l0 < leads; l0 += kMergeThreads / kSmallCell) {
         const uint32_t l = l0 + (threadIdx.x & 31) / kSmallCell;
         const uint2 c = l < leads ? s_lead[l] : make_uint2(0u, 0u);
@@ -617,11 +670,11 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
     CK(cudaMemsetAsync(w.counters, 0, 16 * 4, st));
     CK(cudaMemsetAsync(w.info, 0, 16 * 4, st));
     CK(cudaMemsetAsync(w.role, 0xFF, (size_t)n * 4, st));
-    k_merge_keys<<<(unsigned)blocks, kMergeThreads, 0, st>>>(reinterpret_cast<const float4*>(in_p[0]), in_p[1], n,
-                                                              param_mode, lo[0], lo[1], lo[2], inv, scale_max, w.key);
-    count_launches();
-    CK(cudaGetLastError());
-    k_hist<<<(unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 4), 256, 0, st>>>(w.key, nn, 4, w.hist);
+    uint32_t* three = w.counters + 9;
+    CK(cudaMemsetAsync(three, 1, 4, st));  // (not zero)
+    k_merge_keys<<<(unsigned)std::min<int64_t>(blocks, 152 * 8), kMergeThreads, 0, st>>>(
+        reinterpret_cast<const float4*>(in_p[0]), in_p[1], n, param_mode, lo[0], lo[1], lo[2], inv, scale_max, w.key,
+        w.hist, three);
     count_launches();
     CK(cudaGetLastError());
     for (int p = 0; p < 4; ++p) {  // (key, index) -> A -> B -> A -> B
@@ -630,6 +683,9 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
         if (p == 0)
             k_radix_pass<true, false, false, kSortIpt, true><<<(unsigned)sb, kSortThreads, 0, st>>>(w.key, w.items_a, nullptr, nn, 0, hist,
                                                                              status, w.counters + p, w.info);
+        else if (p == 3)  // nothing to do when three passes sorted the keys
+            k_radix_pass<false, false, true, kSortIpt, true><<<(unsigned)sb, kSortThreads, 0, st>>>(
+                w.items_a, w.items_b, nullptr, nn, 24, hist, status, w.counters + p, w.info, 0xFFFFFFFFu, three);
         else
             k_radix_pass<false, false, false, kSortIpt, true><<<(unsigned)sb, kSortThreads, 0, st>>>(
                 p % 2 ? w.items_a : w.items_b, p % 2 ? w.items_b : w.items_a, nullptr, nn, 8 * p, hist, status,
@@ -637,7 +693,7 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
         count_launches();
         CK(cudaGetLastError());
     }
-    const u64* sorted = w.items_b;
+    const SortedItems sorted{w.items_a, w.items_b, three};
     k_merge_mark<<<(unsigned)blocks, kMergeThreads, 0, st>>>(sorted, n, w.role, w.cells, w.counters + 8, w.info);
     count_launches();
     CK(cudaGetLastError());
