@@ -34,11 +34,12 @@
 // column meets its footprint disc: row_span.)
 //
 // Each radix pass is a single sweep over (key | value) items: a block counts
-// the digits of its 5120 items and publishes those counts at once, ranks the
-// items within each warp with ballots, looks back over earlier blocks (eight
-// at a time) for its global digit offsets, and scatters the items staged in
-// digit order. Every wait on another block or warp is bounded (kMaxSpin polls);
-// on expiry it records IGS_ERR_DEVICE_TIMEOUT, which aborts the frame.
+// the digits of its 5120 items (2048 in depth sorts of up to 778K) and publishes
+// those counts at once, ranks the items within each warp with ballots, looks
+// back over earlier blocks (eight at a time) for its global digit offsets, and
+// scatters the items staged in digit order. Every wait on another block or warp
+// is bounded (kMaxSpin polls); on expiry it records IGS_ERR_DEVICE_TIMEOUT,
+// which aborts the frame.
 #include <algorithm>
 #include <mutex>
 
