@@ -70,6 +70,28 @@ constexpr uint32_t kChunkLeast = 128;
 constexpr int kWalkWarps = 4;              // warps per CTA of the walk kernels (one chunk each)
 constexpr int kWalkUnroll = 8;             // items per lane per round of the counting walks
 
+// With footprint 1: the rectangle r of a kept Gaussian, its rows narrowed to those in which
+// its disc touches a tile (the rows that k_bin_prep finds on its way through them). A disc
+// centred beside the grid reaches the grid only in some of its rectangle's rows; lists of
+// the others too could outgrow the entries, and with them the lists' buffer and the level-2
+// chunks. The rows are consecutive: the half width of row_span falls with the
+// row's distance from the centre, every step of it rounded monotonically. A rectangle that
+// ends before the grid does on both sides holds its centre's column, which the disc meets
+// in every row.
+__device__ __forceinline__ uint2 touched_rows(uint2 r, const float4* __restrict__ disc, int tile, float inv_tile,
+                                              int tiles_x) {
+    if ((r.x & 0xFFFFu) > 0u && (int)(r.y & 0xFFFFu) < tiles_x - 1) return r;
+    const float4 d = *disc;
+    auto none = [&](int y) {
+        const int2 sp = disc_span(d, tile, inv_tile, y);
+        return sp.y < sp.x;
+    };
+    int ya = (int)(r.x >> 16), yb = (int)(r.y >> 16);
+    while (ya < yb && none(ya)) ++ya;  // (a kept Gaussian touches a tile)
+    while (ya < yb && none(yb)) --yb;
+    return make_uint2((r.x & 0xFFFFu) | ((uint32_t)ya << 16), (r.y & 0xFFFFu) | ((uint32_t)yb << 16));
+}
+
 // Depth-digit histograms of all n depth keys, the kept count, and for every kept
 // Gaussian, in each tile row, +1 at its first touched tile and -1 past its last
 // in the (tiles_y+1) x (tiles_x+1) grid (a prefix sum along each row then gives
@@ -78,14 +100,14 @@ constexpr int kWalkUnroll = 8;             // items per lane per round of the co
 // column, then along each row). Each thread has kPrepUnroll Gaussians in flight;
 // the top byte of a view's depths is mostly one value, so a warp whose lanes
 // share it adds its count once instead of 32 times to one shared-memory word.
-// With rowd (the counting-sort route), also +1 at the first row of every kept
-// Gaussian's rectangle and -1 past its last in rowd[tiles_y + 1] (a prefix
+// With rowd (the counting-sort route), also +1 at the first row in which a kept
+// Gaussian touches a tile and -1 past the last one in rowd[tiles_y + 1] (a prefix
 // sum over the rows then gives each tile row's level-1 list length); on the
 // shared-memory grid these sit after the grid's cells.
 constexpr int kPrepUnroll = 4;
-template <bool SMEM_GRID>
+template <bool SMEM_GRID, bool DISCS>
 __global__ void __launch_bounds__(256) k_bin_prep(const uint32_t* __restrict__ depth_key, const uint2* __restrict__ rect,
-                                                  const float4* __restrict__ disc, int tile, int footprint,
+                                                  const float4* __restrict__ disc, int tile,
                                                   const uint32_t* __restrict__ count, uint32_t n, int gx,
                                                   int gy, uint32_t* __restrict__ hist, int32_t* __restrict__ grid,
                                                   int32_t* __restrict__ rowd, uint32_t* __restrict__ info) {
@@ -141,11 +163,12 @@ __global__ void __launch_bounds__(256) k_bin_prep(const uint32_t* __restrict__ d
             if (cnt[u]) {
                 ++kept;
                 const int y0 = r[u].x >> 16, y1 = r[u].y >> 16;
-                if (rowd) {
+                if (rowd && !DISCS) {
                     atomicAdd(&rd[y0], 1);
                     atomicAdd(&rd[y1 + 1], -1);
                 }
-                if (SMEM_GRID && footprint == 0) {  // the rectangle's four corners (a 2D difference)
+                int ya = -1, yb = -1;  // (discs) the first and last row in which it touches a tile
+                if (SMEM_GRID && !DISCS) {  // the rectangle's four corners (a 2D difference)
                     const int x0 = r[u].x & 0xFFFF, x1 = r[u].y & 0xFFFF;
                     atomicAdd(&g[y0 * gx + x0], 1);
                     atomicAdd(&g[y0 * gx + x1 + 1], -1);
@@ -153,10 +176,16 @@ __global__ void __launch_bounds__(256) k_bin_prep(const uint32_t* __restrict__ d
                     atomicAdd(&g[(y1 + 1) * gx + x1 + 1], 1);
                 } else {
                     for (int ty = y0; ty <= y1; ++ty) {  // +1 at the row's first touched tile, -1 past its last
-                        const int2 sp = tile_span(footprint, r[u], disc, i, tile, inv, ty);
+                        const int2 sp = tile_span(DISCS ? 1 : 0, r[u], disc, i, tile, inv, ty);
                         if (sp.y < sp.x) continue;
+                        if (ya < 0) ya = ty;
+                        yb = ty;
                         atomicAdd(&g[ty * gx + sp.x], 1);
                         atomicAdd(&g[ty * gx + sp.y + 1], -1);
+                    }
+                    if (DISCS && rowd && ya >= 0) {
+                        atomicAdd(&rd[ya], 1);
+                        atomicAdd(&rd[yb + 1], -1);
                     }
                 }
             }
@@ -214,15 +243,16 @@ __device__ __forceinline__ void publish_tile_total(unsigned long long* s_total, 
 }
 
 // Row layout of the counting sort, by one block of NT threads once the tile
-// ranges are known (after publish_tile_total). len[y]: the kept Gaussians whose
-// rectangle spans tile row y (prefix of the row differences rowd), the length
-// of row y's level-1 list. rowinfo = [rows] list starts (prefix of len),
-// [rows] first level-2 chunk, [rows] items per level-2 chunk, [1] level-2 chunk
-// total. A row's level-2 chunks take about `target` entries each (kChunkTarget or fewer):
-// target * len / entries items, at least 32, where the row's entries are
-// rowstart[y + 1] - rowstart[y] (rowstart[y]: the first entry of the row's
-// tiles, held in column tiles_x of the grid g; rowstart[rows] = M). Records an
-// error if the chunks exceed max_chunks.
+// ranges are known (after publish_tile_total). len[y]: the length of row y's
+// level-1 list, the kept Gaussians that touch a tile of the row (prefix of the row
+// differences rowd), so that a list has no more items than the row has entries.
+// rowinfo = [rows] list starts (prefix of len), [rows] first level-2 chunk, [rows]
+// items per level-2 chunk, [1] level-2 chunk total. A row's level-2 chunks take about
+// `target` entries each (kChunkTarget or fewer): target * len / entries items, at least
+// 32, where the row's entries are rowstart[y + 1] - rowstart[y] (rowstart[y]: the first
+// entry of the row's tiles, held in column tiles_x of the grid g; rowstart[rows] = M).
+// Records an error if the chunks exceed max_chunks, or the items M (their buffer holds
+// capacity >= M).
 template <int NT>
 __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, const int32_t* g, int gx, uint32_t rows,
                                            uint32_t tiles_x, uint32_t M, uint32_t max_chunks,
@@ -256,7 +286,8 @@ __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, con
     uint32_t base = block_excl_scan<NT>(chunks, s_warp);
     if (threadIdx.x == NT - 1) {
         rowinfo[3 * rows] = base + chunks;
-        if (base + chunks > max_chunks) record_error(info, IGS_ERR_CUDA);  // never expected: chunks are bounded
+        // never expected: both are bounded
+        if (base + chunks > max_chunks || start + items > M) record_error(info, IGS_ERR_CUDA);
     }
     run = lfirst;
     for (uint32_t y = y0; y < y1; ++y) {
@@ -411,7 +442,7 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
 //
 // Two levels, each a counting sort with few buckets:
 //   level 1 places each kept Gaussian, in depth order, into the list of every
-//            tile row its rectangle spans (buckets: rows; items: Gaussian ids);
+//            tile row in which it touches a tile (buckets: rows; items: Gaussian ids);
 //   level 2 places each item of a row, in list order, into every tile of that
 //            row its rectangle spans (buckets: the row's tiles; items: entries).
 // A level counts its chunks' items per bucket (shared memory), scans the counts
@@ -543,6 +574,7 @@ struct DiscRef {
     int tile;
     float inv_tile;
     int footprint;
+    int tiles_x;
 };
 
 using Placer1 = Placer<u64, kStage1>;      // level 1: (column span << 32 | Gaussian id) items
@@ -570,12 +602,13 @@ __device__ __forceinline__ void diff_to_counts(const uint32_t* d, uint32_t B, in
 }
 
 // Level 1, count: for each of its chunks c (grid-stride over warps), a warp adds,
-// for each Gaussian of the chunk, one to every row of its rectangle (as +1 at
-// its first row and -1 past its last, summed along the rows at the end); writes
-// column c of H1 [rows][cmax], and the rectangles in depth order (srect[p] =
-// rect[order[p]]) so that the placement reads them without a gather.
+// for each Gaussian of the chunk, one to every row in which it touches a tile (as +1 at
+// the first and -1 past the last, summed along the rows at the end); writes
+// column c of H1 [rows][cmax], and the rectangles of those rows in depth order (srect[p]:
+// that of order[p]) so that the placement reads them without a gather.
+template <bool DISCS>
 __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* __restrict__ order,
-                                                                const uint2* __restrict__ rect, uint32_t rows,
+                                                                DiscRef disc, uint32_t rows,
                                                                 uint32_t cmax, uint32_t* __restrict__ H1,
                                                                 uint2* __restrict__ srect,
                                                                 const uint32_t* __restrict__ info) {
@@ -599,7 +632,11 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* 
             }
 #pragma unroll
             for (int k = 0; k < kWalkUnroll; ++k) {
-                const uint2 r = g[k] != 0xFFFFFFFFu ? rect[g[k]] : make_uint2(1u << 16, 0u);  // rows 1..0: none
+                uint2 r = make_uint2(1u << 16, 0u);  // rows 1..0: none
+                if (g[k] != 0xFFFFFFFFu) {
+                    r = disc.rect[g[k]];
+                    if (DISCS) r = touched_rows(r, disc.disc + g[k], disc.tile, disc.inv_tile, disc.tiles_x);
+                }
                 ry[k] = (r.x >> 16) | (r.y & 0xFFFF0000u);
                 if (g[k] != 0xFFFFFFFFu) srect[b + k * 32 + lane] = r;  // the placement reads it in order
             }
@@ -620,8 +657,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* 
 
 // Level 1, scan: block y turns row y of H1 (the used chunks' counts) into
 // exclusive offsets in place. The row's total must equal len[y], the list
-// length the row layout was built from (both count the kept Gaussians whose
-// rectangle spans row y); a difference records an error and aborts the frame
+// length the row layout was built from (both count the kept Gaussians that touch
+// a tile of row y); a difference records an error and aborts the frame
 // before any placement. With tile_order, one block more orders the tiles for the
 // blends (order_tiles) while the rows are scanned.
 constexpr int kRowScanThreads = 1024;
@@ -680,7 +717,7 @@ __global__ void __launch_bounds__(kRowScanThreads) k_rows_scan(uint32_t* __restr
 }
 
 // Level 1, place: a warp walks each of its chunks again and puts each Gaussian
-// into the list of every row of its rectangle (R1, rows one after another), as
+// into the list of every row in which it touches a tile (R1, rows one after another), as
 // the item (xa | xb << 16) << 32 | id with the tiles [xa, xb] it touches in
 // that row ((1, 0): none), so that level 2 reads its items without a gather.
 __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_place(const uint32_t* __restrict__ order,
@@ -1129,17 +1166,14 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
     const bool few = depth_sort_tile(n) != kSortTile;
     // 0. depth-digit histograms; footprint rows -> per-tile counts -> ranges, tile-digit histograms
     const int prep_blocks = (int)std::min<int64_t>(ceil_div(n, 256), 152 * 4);
-    if ((int64_t)gx * gy <= kGridSmemCells)
-        CK(launch_pdl(k_bin_prep<true>, dim3(prep_blocks), dim3(256), (size_t)(gx * gy + (walk ? gy : 0)) * 4, st,
-            f.depth_key, reinterpret_cast<const uint2*>(f.rect), reinterpret_cast<const float4*>(f.disc), f.tile,
-            footprint, f.count, nn, gx, gy, s.hist, s.grid, rowd, f.info));
-    else
-        CK(launch_pdl(k_bin_prep<false>, dim3(prep_blocks), dim3(256), 0, st, f.depth_key, reinterpret_cast<const uint2*>(f.rect),
-                                                       reinterpret_cast<const float4*>(f.disc), f.tile, footprint,
-                                                       f.count, nn, gx, gy, s.hist, s.grid, rowd, f.info));
+    const bool small_grid = (int64_t)gx * gy <= kGridSmemCells;
+    const auto prep = footprint ? (small_grid ? k_bin_prep<true, true> : k_bin_prep<false, true>)
+                                : (small_grid ? k_bin_prep<true, false> : k_bin_prep<false, false>);
+    CK(launch_pdl(prep, dim3(prep_blocks), dim3(256), small_grid ? (size_t)(gx * gy + (walk ? gy : 0)) * 4 : 0, st,
+                  f.depth_key, reinterpret_cast<const uint2*>(f.rect), reinterpret_cast<const float4*>(f.disc), f.tile,
+                  f.count, nn, gx, gy, s.hist, s.grid, rowd, f.info));
     count_launches();
     CK(cudaGetLastError());
-    const bool small_grid = (int64_t)gx * gy <= kGridSmemCells;
     if (small_grid) {
         // the depth sort's first pass, then, beside it, the tile ranges by one block (k_tiles_small was 12 to 16 us of
         // every frame's chain when it stood before the pass: frames of 200K and of 1M Gaussians 166 and 352 us,
@@ -1179,14 +1213,16 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
 
         const uint2* rect = reinterpret_cast<const uint2*>(f.rect);
         const uint2* rg = reinterpret_cast<const uint2*>(f.ranges);
-        CK(launch_pdl(k_rows_count, dim3(walk_blocks((const void*)k_rows_count, count1, cmax)), dim3(32 * kWalkWarps), count1, st, f.order, rect, rows, cmax, s.walk_h1, s.walk_rect, f.info));
+        const DiscRef disc{rect, reinterpret_cast<const float4*>(f.disc), f.tile, 1.0f / (float)f.tile, footprint,
+                           f.tiles_x};
+        const auto rows_count = footprint ? k_rows_count<true> : k_rows_count<false>;
+        CK(launch_pdl(rows_count, dim3(walk_blocks((const void*)rows_count, count1, cmax)), dim3(32 * kWalkWarps), count1, st, f.order, disc, rows, cmax, s.walk_h1, s.walk_rect, f.info));
         count_launches();
         CK(cudaGetLastError());
         CK(launch_pdl(k_rows_scan, dim3(rows + (s.tile_order ? 1 : 0)), dim3(kRowScanThreads), 0, st, s.walk_h1, cmax,
                       s.walk_len, f.info, rows, rg, (uint32_t)tiles, s.tile_order));
         count_launches();
         CK(cudaGetLastError());
-        const DiscRef disc{rect, reinterpret_cast<const float4*>(f.disc), f.tile, 1.0f / (float)f.tile, footprint};
         CK(launch_pdl(k_rows_place, dim3(walk_blocks((const void*)k_rows_place, place1, cmax)), dim3(32 * kWalkWarps), place1, st, f.order, s.walk_rect, disc, rows, cmax, s.walk_h1, s.walk_len,
                                                                 s.walk_rows, R1, f.info));
         count_launches();
