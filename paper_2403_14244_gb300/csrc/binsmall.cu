@@ -11,8 +11,11 @@
 //   k_small_place  one CTA per strip of up to eight tiles of a tile row: the strip's tile
 //                  ranges and, in depth order, the entries of its tiles, from the row's
 //                  bitmap (up to kRankMax Gaussians: from all rectangles).
-// 4,096 Gaussians on 256 x 256 pixels: 14 us against 90 for the general route; a whole frame of
-// them 28 us against 90. 20,000 on 320 x 240: 24 us against 84.
+// 4,096 Gaussians on 256 x 256 pixels: 12 us against 41 for the general route; 16,384: 22 against
+// 45. The entries per tile row, which give a strip its first slot, are summed by the merge: with
+// the parts of every 256 Gaussians added up again by every strip, 32,768 Gaussians at 3840 x 2160
+// took 150 us with 16-pixel tiles and 632 with 8-pixel tiles, now 119 and 396 (and the general
+// route takes the latter: bin_small_ok).
 // Writes what launch_bin_sort writes: order, ranges, vals and the status words (the
 // same values: the stable depth order, rectangles row by row).
 #include <mutex>
@@ -99,7 +102,7 @@ __global__ void __launch_bounds__(kRankThreads) k_small_rank(const uint32_t* __r
 
 // Block c sorts Gaussians [1024 c, 1024 c + 1024) by (key, index): a bitonic network,
 // one Gaussian per thread, exchanges within a warp by shuffles. skey holds whole chunks
-// (past the end: the largest key). The row bitmaps of the merge are zeroed on the way.
+// (past the end: the largest key). The row bitmaps and totals of the merge are zeroed on the way.
 __global__ void __launch_bounds__(kChunk) k_small_sort(const uint32_t* __restrict__ key, uint32_t n,
                                                        uint32_t* __restrict__ skey, uint32_t* __restrict__ sid,
                                                        uint32_t* __restrict__ bits, uint32_t words) {
@@ -136,15 +139,15 @@ __global__ void __launch_bounds__(kChunk) k_small_sort(const uint32_t* __restric
 // time, and a thread searches four at once; a warp's Gaussians are neighbours in their
 // chunk's order, so its lanes search nearly the same places. Every kept rectangle then
 // sets its rank's bit in the zeroed bitmap of each tile row it spans (row_words words
-// a row), and block b writes the entries of its Gaussians per tile row to
-// row_part[b][rows].
+// a row), and the block adds the entries of its Gaussians per tile row to the zeroed
+// row_total[rows] (below 2^32: at most kBinSmallMax rectangles of 2048 tiles a row).
 __global__ void __launch_bounds__(kMergeThreads) k_small_merge(const uint32_t* __restrict__ skey,
                                                                const uint32_t* __restrict__ sid, uint32_t n,
                                                                const uint2* __restrict__ rect,
                                                                const uint32_t* __restrict__ count,
                                                                uint32_t* __restrict__ order,
                                                                uint2* __restrict__ srect, uint32_t* __restrict__ bits,
-                                                               uint32_t row_words, uint32_t* __restrict__ row_part,
+                                                               uint32_t row_words, uint32_t* __restrict__ row_total,
                                                                uint32_t rows) {
     pdl_wait();
     __shared__ uint32_t s_row[kBinSmallRows];
@@ -191,7 +194,8 @@ __global__ void __launch_bounds__(kMergeThreads) k_small_merge(const uint32_t* _
         }
     }
     __syncthreads();
-    for (uint32_t y = threadIdx.x; y < rows; y += kMergeThreads) row_part[(size_t)blockIdx.x * rows + y] = s_row[y];
+    for (uint32_t y = threadIdx.x; y < rows; y += kMergeThreads)
+        if (s_row[y]) atomicAdd(&row_total[y], s_row[y]);
 }
 
 __device__ __forceinline__ u64 block_sum64(u64 v, u64* s_part) {
@@ -255,15 +259,15 @@ __device__ __forceinline__ void small_status(const uint32_t* __restrict__ key, u
 // (from the row's bitmap (BITS) or from the rectangles themselves), then those of them
 // that meet the strip. On the way the block counts the entries of each of its tiles, of
 // the row's tiles before the strip, and of the rows before y (its first slot) and of the
-// frame (the capacity check): from row_part[parts][tiles_y], or again from the
+// frame (the capacity check): from row_total[tiles_y], or again from the
 // rectangles. Then every warp walks a part of the list and writes its tiles' entries.
 // A strip met by more than kListMax rectangles is listed and placed again in shorter
 // rounds. Block (tiles_y, 0) writes the status words.
 template <bool BITS>
 __global__ void __launch_bounds__(kPlaceThreads) k_small_place(
     const uint32_t* __restrict__ order, const uint2* __restrict__ srect, const uint32_t* __restrict__ key,
-    const uint32_t* __restrict__ bits, uint32_t row_words, const uint32_t* __restrict__ row_part, uint32_t parts,
-    uint32_t n, uint32_t tiles_x, uint32_t tiles_y, uint32_t per, uint64_t capacity, uint2* __restrict__ ranges,
+    const uint32_t* __restrict__ bits, uint32_t row_words, const uint32_t* __restrict__ row_total, uint32_t n,
+    uint32_t tiles_x, uint32_t tiles_y, uint32_t per, uint64_t capacity, uint2* __restrict__ ranges,
     uint32_t* __restrict__ vals, uint32_t* __restrict__ tile_order, uint32_t* __restrict__ info) {
     pdl_wait();
     constexpr uint32_t kEach = BITS ? kEachBits : kEachRects;
@@ -279,10 +283,10 @@ __global__ void __launch_bounds__(kPlaceThreads) k_small_place(
     if (threadIdx.x < kStrip) s_cnt[threadIdx.x] = 0u;
     u64 before = 0, total = 0;
     if constexpr (BITS) {
-        for (uint32_t i = threadIdx.x; i < parts * tiles_y; i += kPlaceThreads) {
-            const uint32_t v = row_part[i];
+        for (uint32_t i = threadIdx.x; i < tiles_y; i += kPlaceThreads) {
+            const uint32_t v = row_total[i];
             total += v;
-            if (i % tiles_y < y) before += v;
+            if (i < y) before += v;
         }
     } else {
         for (uint32_t p = threadIdx.x; p < n; p += kPlaceThreads) {
@@ -475,7 +479,8 @@ static cudaError_t place_opt_in(int bytes) {
 }
 
 bool bin_small_ok(const igs_frame& f, int footprint) {
-    return footprint == 0 && f.n > 0 && f.n <= kBinSmallMax && f.sort_chunks > 0 && f.tiles_y <= kBinSmallRows;
+    return footprint == 0 && f.n > 0 && f.n <= kBinSmallMax && f.sort_chunks > 0 && f.tiles_y <= kBinSmallRows &&
+           f.n * f.tiles_x * f.tiles_y <= kBinSmallCells;
 }
 
 cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStream_t st) {
@@ -486,22 +491,22 @@ cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStrea
     uint2* srect = s.walk_rect;
     // skey: the 8 n bytes of ditems_a hold n rounded up to 1024 words above kRankMax Gaussians
     uint32_t *skey = reinterpret_cast<uint32_t*>(s.ditems_a), *sid = reinterpret_cast<uint32_t*>(s.ditems_b);
-    // the row bitmaps and row parts: 4 (n / 32 + n / 256 + 2) bytes per tile row of the 4 walk_chunks
+    // the row bitmaps and, after them, the rows' totals: 4 (n / 32 + 2) bytes per tile row of the 4 walk_chunks
     // bytes per row of walk_h1 (at least 32 KB up to kBinSmallRows rows)
-    const uint32_t row_words = (uint32_t)ceil_div(f.n, 32), parts = (uint32_t)ceil_div(f.n, kMergeThreads);
-    uint32_t *bits = s.walk_h1, *row_part = s.walk_h1 + (size_t)row_words * ty;
+    const uint32_t row_words = (uint32_t)ceil_div(f.n, 32);
+    uint32_t *bits = s.walk_h1, *row_total = s.walk_h1 + (size_t)row_words * ty;
     const bool rank = f.n <= kRankMax;
     if (rank) {
         CK(launch_pdl(k_small_rank, dim3((unsigned)ceil_div(f.n, 32)), dim3(kRankThreads), 0, st, f.depth_key, rect,
                       f.count, n, f.order, srect));
     } else {
-        if ((int64_t)row_words + parts > s.walk_chunks) return cudaErrorInvalidValue;  // (never: bin_small_ok)
+        if ((int64_t)row_words + 1 > s.walk_chunks) return cudaErrorInvalidValue;  // (never: bin_small_ok)
         CK(launch_pdl(k_small_sort, dim3((unsigned)ceil_div(f.n, kChunk)), dim3(kChunk), 0, st, f.depth_key, n, skey,
-                      sid, bits, row_words * ty));
+                      sid, bits, (row_words + 1) * ty));
         count_launches();
         CK(cudaGetLastError());
-        CK(launch_pdl(k_small_merge, dim3(parts), dim3(kMergeThreads), 0, st, skey, sid, n, rect, f.count, f.order,
-                      srect, bits, row_words, row_part, ty));
+        CK(launch_pdl(k_small_merge, dim3((unsigned)ceil_div(f.n, kMergeThreads)), dim3(kMergeThreads), 0, st, skey, sid,
+                      n, rect, f.count, f.order, srect, bits, row_words, row_total, ty));
     }
     count_launches();
     CK(cudaGetLastError());
@@ -511,8 +516,8 @@ cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStrea
     const size_t smem = (size_t)(kListMax + (rank ? kEachRects : kEachBits) * kPlaceThreads) * 4;
     if (smem > 40 * 1024) CK(place_opt_in((int)smem));
     CK(launch_pdl(rank ? k_small_place<false> : k_small_place<true>, dim3(ty + 1, (unsigned)ceil_div(f.tiles_x, per)),
-                  dim3(kPlaceThreads), smem, st, f.order, srect, f.depth_key, bits, row_words, row_part, parts, n, tx, ty,
-                  per, (uint64_t)f.capacity,
+                  dim3(kPlaceThreads), smem, st, f.order, srect, f.depth_key, bits, row_words, row_total, n, tx, ty, per,
+                  (uint64_t)f.capacity,
                   reinterpret_cast<uint2*>(f.ranges), f.vals, s.tile_order, f.info));
     count_launches();
     CK(cudaGetLastError());

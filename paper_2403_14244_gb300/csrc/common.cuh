@@ -343,12 +343,20 @@ struct SortScratch {
 };
 SortScratch sort_scratch(const igs_frame& f);
 // The binning of few Gaussians in two or three launches (binsmall.cu): whether a frame takes it, and
-// its launches. The line lies where the two routes meet: 16384 Gaussians take 21-23 us against 82-96 (16-
-// and 32-pixel tiles, 320 x 240 to 1920 x 1080 pixels), 32768 30-33 against 86-97, 65536 54-58
-// against 89-102, 98304 89-95 against 92-102; with 8-pixel tiles at 1297 x 840, 32768 88 against 149,
-// 65536 150 against 168, 98304 224 against 186. (The pieces of the small route grow with n^2 / 1024 and
-// n times the strips.) More tile rows than kBinSmallRows would not fit the merge's row counters.
-constexpr int64_t kBinSmallMax = 65536;
+// its launches. Its pieces grow with n^2 / 1024 (the merge) and with n times the strips (every strip goes
+// over its row's bitmap), so the line is one in n and one in n times the tiles, where the routes meet (igs_bin_sort
+// alone, us, small : general):
+//   tile, pixels       16384        32768        49152        65536
+//   16, 256 x 256       22 : 45      33 : 48      47 : 49      59 : 51
+//   32, 1920 x 1080     21 : 55      30 : 57      43 : 59      53 : 61
+//   16, 1920 x 1080     34 : 73      48 : 75      67 : 78      82 : 81
+//   16, 3840 x 2160     82 : 155    119 : 171    158 : 187    196 : 194
+//    8, 3840 x 2160    275 : 299    396 : 329    519 : 366    642 : 392
+// With four times the scale: 16 pixels at 3840 x 2160 and 49152 263 : 357, 32 pixels at 1920 x 1080 and
+// 65536 106 : 70 (lists past kListMax items are walked again); 256 x 256 and 49152 88 : 51.
+// More tile rows than kBinSmallRows would not fit the merge's row counters.
+constexpr int64_t kBinSmallMax = 49152;
+constexpr int64_t kBinSmallCells = (int64_t)1 << 31;  // Gaussians x tiles
 constexpr int64_t kBinSmallRows = 512;
 bool bin_small_ok(const igs_frame& f, int footprint);
 cudaError_t launch_bin_small(const igs_frame& f, const SortScratch& s, cudaStream_t st);
