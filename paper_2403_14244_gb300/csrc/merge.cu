@@ -16,10 +16,11 @@
 //                    the position of a cell of more than eight in a list
 //   k_merge_count    per block of Gaussians: how many are written, and which
 //   k_merge_scan     one CTA: each block's first output slot, the total
-//   k_merge_cells    a warp per merged cell of more than eight members
 //   k_merge_write    per block of Gaussians: output slots; kept Gaussians copy
 //                    parameters and moments (colour rows cooperatively); the
-//                    smaller cells led there are merged, eight lanes a cell
+//                    smaller cells led there are merged, eight lanes a cell; and
+//                    in blocks of their own the merged cells of more than eight
+//                    members, a warp each
 // A merged Gaussian: FP32, compensated sums over the members in index order,
 // means relative to the first member, zero moments.
 //
@@ -296,7 +297,7 @@ __device__ __forceinline__ void write_merged(MergeOut out, size_t d, float4 m0, 
 
 // A merged cell of at most kSmallCell members (sorted items from p0 on, output slot d;
 // have: there is one) per eight lanes, four to a warp: lane j of the eight holds its
-// member j, and every sum adds the members' terms in index order, as k_merge_cells
+// member j, and every sum adds the members' terms in index order, as merge_large
 // does; a colour row is read and written by the eight lanes together.
 template <int C>
 __device__ __forceinline__ void merge_small(const MergeArrays& in, const MergeOut& out, int64_t n, int param_mode,
@@ -391,24 +392,16 @@ __device__ __forceinline__ void merge_small(const MergeArrays& in, const MergeOu
     }
 }
 
-// Merged cells of more than kSmallCell members, one to a warp (a grid-stride loop over
-// the list): lane j holds member j of each run of 32 (index order), and every sum adds
+// Merged cells of more than kSmallCell members, one to a warp (warps first, first + warps, ...
+// of the list): lane j holds member j of each run of 32 (index order), and every sum adds
 // the members' terms in index order; colour coefficient c is lane c mod 32's.
 template <int C>
-__global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, MergeOut out, int64_t n,
-                                                               int param_mode, SortedItems sorted,
-                                                               const uint32_t* __restrict__ cells,
-                                                               const uint32_t* __restrict__ n_cells,
-                                                               const uint32_t* __restrict__ blk,
-                                                               const uint32_t* __restrict__ emit_bits,
-                                                               const uint32_t* __restrict__ info) {
-    pdl_trigger();  // k_merge_write needs nothing written here
-    if (info[kInfoAbort]) return;
-    const uint32_t total = *n_cells;
-    const u64* __restrict__ items = sorted.get();
+__device__ __forceinline__ void merge_large(const MergeArrays& in, const MergeOut& out, int64_t n, int param_mode,
+                                            const u64* __restrict__ items, const uint32_t* __restrict__ cells,
+                                            uint32_t total, const uint32_t* __restrict__ blk,
+                                            const uint32_t* __restrict__ emit_bits, uint32_t first, uint32_t warps) {
     const int lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * (kMergeThreads / 32);
-    for (uint32_t g = blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5); g < total; g += warps) {
+    for (uint32_t g = first; g < total; g += warps) {
         const int64_t p0 = cells[g];
         const uint32_t key = (uint32_t)(items[p0] >> 32);
         const size_t d = leader_slot((uint32_t)items[p0], lane & 7, blk, emit_bits);
@@ -530,25 +523,33 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_cells(MergeArrays in, M
 // them, a warp per cell 330 (158 as four cells to a warp; as a kernel beside this one
 // no less in all: its reads then wait on the copies'). Four blocks per SM and four
 // accesses in flight: with two 23 us more, five blocks 37, three 43.
-// Runs beside k_merge_cells, whose launch it follows without waiting for it. Its last
-// block ends after k_merge_cells, so that what follows in the stream finds both.
+// The first cell_blocks blocks merge the larger cells instead, a warp each, under the
+// copies of the others (one after the other, 3M Gaussians on 32 and 64 cells an axis took
+// 1006 and 830 us in all, so 727 and 695).
 template <int C>
 __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in, MergeOut out, int64_t n, int param_mode,
                                                                SortedItems sorted, const uint32_t* __restrict__ role,
                                                                const uint32_t* __restrict__ blk,
+                                                               const uint32_t* __restrict__ emit_bits,
+                                                               const uint32_t* __restrict__ cells,
+                                                               const uint32_t* __restrict__ n_cells,
+                                                               uint32_t cell_blocks,
                                                                const uint32_t* __restrict__ info) {
-    if (info[kInfoAbort]) {
-        if (blockIdx.x == gridDim.x - 1) pdl_wait();
+    if (info[kInfoAbort]) return;
+    if (blockIdx.x < cell_blocks) {
+        merge_large<C>(in, out, n, param_mode, sorted.get(), cells, *n_cells, blk, emit_bits,
+                       blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5), cell_blocks * (kMergeThreads / 32));
         return;
     }
     __shared__ uint32_t s_warp[kMergeThreads / 32];
     __shared__ uint32_t s_dst[kMergeThreads];  // output slot of a kept Gaussian, else ~0
     __shared__ uint2 s_lead[kMergeThreads];    // small cells led here: start of the items, output slot
     __shared__ uint32_t s_leads;
-    const int64_t i0 = (int64_t)blockIdx.x * kMergeThreads, i = i0 + threadIdx.x;
+    const uint32_t b = blockIdx.x - cell_blocks;
+    const int64_t i0 = (int64_t)b * kMergeThreads, i = i0 + threadIdx.x;
     const uint32_t rl = i < n ? role[i] : kRoleGone;
     if (threadIdx.x == 0) s_leads = 0u;
-    const uint32_t slot = blk[blockIdx.x] + block_excl_scan<kMergeThreads>(rl != kRoleGone ? 1u : 0u, s_warp);
+    const uint32_t slot = blk[b] + block_excl_scan<kMergeThreads>(rl != kRoleGone ? 1u : 0u, s_warp);
     s_dst[threadIdx.x] = rl == kRoleKept ? slot : 0xFFFFFFFFu;
     const size_t d = slot, s = (size_t)i;
     if (rl == kRoleKept) {
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in
     T* ovc = reinterpret_cast<T*>(out.v_col);
     constexpr int U = 4;  // accesses of each array in flight per thread
     for (int q0 = threadIdx.x; q0 < nr * CV; q0 += U * kMergeThreads) {
-        T a[U], b[U], c[U];
+        T a[U], m[U], v[U];
         size_t dst[U];
         bool on[U];
 #pragma unroll
@@ -586,16 +587,16 @@ __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in
             if (on[u]) {
                 const size_t src = (size_t)(i0 + j) * CV + f;
                 a[u] = icol[src];
-                b[u] = imc[src];
-                c[u] = ivc[src];
+                m[u] = imc[src];
+                v[u] = ivc[src];
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (on[u]) {
                 ocol[dst[u]] = a[u];
-                omc[dst[u]] = b[u];
-                ovc[dst[u]] = c[u];
+                omc[dst[u]] = m[u];
+                ovc[dst[u]] = v[u];
             }
     }
     const uint32_t leads = s_leads;
@@ -606,7 +607,6 @@ __global__ void __launch_bounds__(kMergeThreads, 4) k_merge_write(MergeArrays in
         merge_small<C>(in, out, n, param_mode, items, c.x, c.y, l < leads);
         __syncwarp();
     }
-    if (blockIdx.x == gridDim.x - 1) pdl_wait();
 }
 
 // Work layout (all 256-byte aligned pieces).
@@ -708,18 +708,14 @@ cudaError_t launch_merge(const float* const in_p[3], const float* const in_m[3],
                    in_m[1], in_m[2], reinterpret_cast<const float4*>(in_v[0]), in_v[1], in_v[2]};
     MergeOut out{reinterpret_cast<float4*>(out_p[0]), out_p[1], out_p[2], reinterpret_cast<float4*>(out_m[0]),
                  out_m[1], out_m[2], reinterpret_cast<float4*>(out_v[0]), out_v[1], out_v[2]};
-    // at most two blocks per SM (half its registers): k_merge_write runs in what is left
+    // at most two blocks per SM, half of it: the copies run in the rest
     const unsigned cell_blocks =
         (unsigned)std::min<int64_t>(ceil_div(n, (kSmallCell + 1) * kMergeThreads / 32), 152 * 2);
     switch (C) {  // colour floats per Gaussian: a compile-time row length for the cooperative copies
 #define IGS_MERGE_C(CC)                                                                                             \
     case CC:                                                                                                        \
-        k_merge_cells<CC><<<cell_blocks, kMergeThreads, 0, st>>>(in, out, n, param_mode, sorted, w.cells,            \
-                                                                 w.counters + 8, w.blk, emit_bits, w.info);         \
-        count_launches();                                                                                           \
-        CK(cudaGetLastError());                                                                                     \
-        CK(launch_pdl(k_merge_write<CC>, dim3((unsigned)blocks), dim3(kMergeThreads), 0, st, in, out, n, param_mode, \
-                      sorted, (const uint32_t*)w.role, (const uint32_t*)w.blk, (const uint32_t*)w.info));           \
+        k_merge_write<CC><<<(unsigned)(cell_blocks + blocks), kMergeThreads, 0, st>>>(                              \
+            in, out, n, param_mode, sorted, w.role, w.blk, emit_bits, w.cells, w.counters + 8, cell_blocks, w.info); \
         count_launches();                                                                                           \
         CK(cudaGetLastError());                                                                                     \
         break;
