@@ -107,16 +107,17 @@ __global__ void __launch_bounds__(1024) k_hist_to_offsets(uint32_t* __restrict__
 // COUNTS: digit_base holds the digits' raw counts, and each block forms the offsets.
 // AHEAD (a frame's first pass): the next launch may start before this one ends
 // (k_tiles_small, which needs none of its results and sets the abort flag meanwhile:
-// no block looks at it).
+// no block looks at it); it finds the word `started` set.
 template <bool IN_KEYS32, bool OUT_VALS, bool SKIPPABLE = false, int IPT = kSortIpt, bool COUNTS = false,
           bool AHEAD = false>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_pass(
     const void* __restrict__ in_, void* __restrict__ out_, const uint32_t* __restrict__ d_count, uint32_t count_host,
     int shift, const uint32_t* __restrict__ digit_base, uint32_t* __restrict__ status,
     uint32_t* __restrict__ block_counter, uint32_t* __restrict__ info, uint32_t silent_blk = 0xFFFFFFFFu,
-    const uint32_t* __restrict__ skip_flag = nullptr, uint32_t* __restrict__ skip_vals = nullptr) {
+    const uint32_t* __restrict__ skip_flag = nullptr, uint32_t* __restrict__ skip_vals = nullptr,
+    uint32_t* __restrict__ started = nullptr) {
     pdl_wait();
-    if (AHEAD) pdl_trigger();
+    if (AHEAD) pdl_ahead(started);
     constexpr int kTile = kSortThreads * IPT;  // items per block
     if (SKIPPABLE && !skip_vals && *skip_flag) return;
     {

@@ -71,10 +71,30 @@ __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + 
 // its writes are visible. Without the launch attribute pdl_wait() is a no-op.
 // (Kernels do not trigger their successors early, but where a successor has work
 // that needs nothing of them: resident waiting CTAs slowed the predecessors' last
-// waves, measured. Such a successor calls pdl_wait() in one block before it ends,
-// so that what follows it in the stream follows both.)
+// waves, measured.)
+//
+// Such a pair: the predecessor, once it may read what came before it (after its own
+// pdl_wait(), or at its start without the launch attribute), calls pdl_ahead(), whose
+// first block releases a word that was zero, and triggers. The successor calls
+// pdl_behind() before it touches memory: it acquires the word, which makes visible what
+// came before the predecessor (the trigger alone promises nothing of the kind), or waits
+// for the whole predecessor if it does not find it set. And it calls pdl_wait() in one
+// block before it ends, so that what follows it in the stream follows both. Data that is
+// read this way is read by coherent loads (ld_cg).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_ahead(uint32_t* started) {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(started), "r"(1u) : "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_behind(const uint32_t* started) {  // every thread of the block calls it
+    uint32_t set = 1u;
+    if (threadIdx.x == 0)
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(set) : "l"(started) : "memory");
+    if (__syncthreads_or(set == 0u)) pdl_wait();
+}
+template <typename T>
+__device__ __forceinline__ T ld_cg(const T* p) { return __ldcg(p); }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args&&... args) {

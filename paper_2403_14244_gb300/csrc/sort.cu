@@ -263,7 +263,7 @@ __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, con
     const uint32_t per = (rows + NT - 1) / NT;
     const uint32_t y0 = min(rows, threadIdx.x * per), y1 = min(rows, y0 + per);
     uint32_t dsum = 0;
-    for (uint32_t y = y0; y < y1; ++y) dsum += (uint32_t)rowd[y];
+    for (uint32_t y = y0; y < y1; ++y) dsum += (uint32_t)ld_cg(rowd + y);
     const uint32_t lfirst = block_excl_scan<NT>(dsum, s_warp);  // modulo 2^32: the differences' prefix
     // entries per chunk: kChunkTarget, fewer where M has less than kWalkFill such chunks, as far as
     // max_chunks allows: a row has at most 33/32 entries / target + 1 chunks (a chunk's items, 32 or
@@ -272,7 +272,7 @@ __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, con
     const uint32_t target = min(kChunkTarget, max(kChunkLeast, M / fill + 1));
     uint32_t items = 0, chunks = 0, run = lfirst;
     for (uint32_t y = y0; y < y1; ++y) {
-        run += (uint32_t)rowd[y];
+        run += (uint32_t)ld_cg(rowd + y);
         const uint32_t ly = run;
         const uint64_t entries = rowstart(y + 1) - rowstart(y);
         const uint32_t size =
@@ -291,7 +291,7 @@ __device__ __forceinline__ void row_layout(const int32_t* __restrict__ rowd, con
     }
     run = lfirst;
     for (uint32_t y = y0; y < y1; ++y) {
-        run += (uint32_t)rowd[y];
+        run += (uint32_t)ld_cg(rowd + y);
         const uint32_t size = rowinfo[2 * rows + y];
         rowinfo[y] = start;
         rowinfo[rows + y] = base;
@@ -356,8 +356,9 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
                                                                     uint32_t* __restrict__ info, uint64_t capacity,
                                                                     const int32_t* __restrict__ rowd,
                                                                     uint32_t max_chunks, uint32_t* __restrict__ len,
-                                                                    uint32_t* __restrict__ rowinfo) {
-    // (no wait: it runs beside the depth sort's first pass, which started after the kernel that counted)
+                                                                    uint32_t* __restrict__ rowinfo,
+                                                                    const uint32_t* __restrict__ started) {
+    pdl_behind(started);  // it runs beside the depth sort's first pass, which started after the kernel that counted
     extern __shared__ int32_t s_g[];
     __shared__ uint32_t s_h[8][kRadix];
     __shared__ uint32_t s_warp[kTilesSmallThreads / 32];
@@ -365,15 +366,15 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
     if (threadIdx.x == 0) s_total = 0ull;
     const int gx = tiles_x + 1, cells = gx * (tiles_y + 1);
     const int tid = threadIdx.x;
-    for (int k = tid; k < cells; k += blockDim.x) s_g[k] = grid[k];
-    for (int k = tid; k < 4 * kRadix; k += blockDim.x) (&s_h[0][0])[k] = hist[k];          // depth counts
+    for (int k = tid; k < cells; k += blockDim.x) s_g[k] = ld_cg(grid + k);
+    for (int k = tid; k < 4 * kRadix; k += blockDim.x) (&s_h[0][0])[k] = ld_cg(hist + k);  // depth counts
     for (int k = tid; k < 4 * kRadix; k += blockDim.x) (&s_h[4][0])[k] = 0;                // tile counts
     __syncthreads();
     if (tid < 32) {  // skip the top depth pass: at most one top byte other than the culled 0xFF, no wrap
         uint32_t nz = 0;
         for (int b = tid; b < kRadix - 1; b += 32) nz += s_h[3][b] != 0u;
         nz = __reduce_add_sync(0xffffffffu, nz);
-        if (tid == 0) info[kInfoSkipTop] = (nz <= 1u && info[kInfoKeyWrap] == 0u) ? 1u : 0u;
+        if (tid == 0) info[kInfoSkipTop] = (nz <= 1u && ld_cg(info + kInfoKeyWrap) == 0u) ? 1u : 0u;
     }
     if (diff2d) {  // rectangles were added as 2D differences: a prefix down each column first
         for (int x = tid; x < tiles_x; x += blockDim.x) {
@@ -1083,6 +1084,8 @@ SortScratch sort_scratch(const igs_frame& f) {
 // with one silent block (igs_debug_silence_lookback_once).
 std::atomic<int> g_silence_next{0};
 
+constexpr int kStartedWord = 15;  // of the counters: set once the first pass has started (pdl_ahead)
+
 // The passes of a frame's depth sort. On a small grid the first one is launched before
 // k_tiles_small, from raw digit counts, and k_tiles_small decides the top-pass skip.
 template <int IPT>
@@ -1091,7 +1094,7 @@ static cudaError_t launch_first_pass(const igs_frame& f, const SortScratch& s, c
     const cudaError_t e = launch_pdl(k_radix_pass<true, false, false, IPT, true, true>, blocks, threads, 0, st,
                                      f.depth_key, s.ditems_a, nullptr, (uint32_t)f.n, 0, s.hist, s.status_depth,
                                      s.counters + 0, f.info, g_silence_next.exchange(0) ? 1u : 0xFFFFFFFFu, nullptr,
-                                     nullptr);
+                                     nullptr, s.counters + kStartedWord);
     count_launches();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1108,22 +1111,22 @@ static cudaError_t launch_depth_sort(const igs_frame& f, const SortScratch& s, b
         if (p == 0)
             e = launch_pdl(k_radix_pass<true, false, false, IPT>, blocks, threads, 0, st, f.depth_key, s.ditems_a, nullptr,
                            nn, 0, hist, status, s.counters + 0, f.info, g_silence_next.exchange(0) ? 1u : 0xFFFFFFFFu,
-                           nullptr, nullptr);
+                           nullptr, nullptr, nullptr);
         else if (p == 1)
             e = launch_pdl(k_radix_pass<false, false, false, IPT>, blocks, threads, 0, st, s.ditems_a, s.ditems_b, nullptr,
-                           nn, 8, hist, status, s.counters + 1, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+                           nn, 8, hist, status, s.counters + 1, f.info, 0xFFFFFFFFu, nullptr, nullptr, nullptr);
         else if (p == 2 && small_grid)  // writes the order itself when the top pass is skipped
             e = launch_pdl(k_radix_pass<false, false, true, IPT>, blocks, threads, 0, st, s.ditems_b, s.ditems_a, nullptr,
-                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, skip, f.order);
+                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, skip, f.order, nullptr);
         else if (p == 2)
             e = launch_pdl(k_radix_pass<false, false, false, IPT>, blocks, threads, 0, st, s.ditems_b, s.ditems_a, nullptr,
-                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+                           nn, 16, hist, status, s.counters + 2, f.info, 0xFFFFFFFFu, nullptr, nullptr, nullptr);
         else if (small_grid)  // nothing to do when the top pass is skipped
             e = launch_pdl(k_radix_pass<false, true, true, IPT>, blocks, threads, 0, st, s.ditems_a, f.order, nullptr, nn,
-                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, skip, nullptr);
+                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, skip, nullptr, nullptr);
         else
             e = launch_pdl(k_radix_pass<false, true, false, IPT>, blocks, threads, 0, st, s.ditems_a, f.order, nullptr, nn,
-                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, nullptr, nullptr);
+                           24, hist, status, s.counters + 3, f.info, 0xFFFFFFFFu, nullptr, nullptr, nullptr);
         count_launches();
         if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1182,7 +1185,7 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
         CK(launch_pdl(k_tiles_small, dim3(1), dim3(kTilesSmallThreads), (size_t)gx * gy * 4, st,
                       (const int32_t*)s.grid, f.tiles_x, f.tiles_y, tp, footprint == 0 ? 1 : 0,
                       reinterpret_cast<uint2*>(f.ranges), s.hist, f.info, (uint64_t)cap, (const int32_t*)rowd, max2,
-                      s.walk_len, s.walk_rows));
+                      s.walk_len, s.walk_rows, (const uint32_t*)s.counters + kStartedWord));
         count_launches();
         CK(cudaGetLastError());
     } else {
@@ -1260,11 +1263,11 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
         if (p == tp - 1)
             CK(launch_pdl(k_radix_pass<false, true>, dim3((unsigned)bc), dim3(kSortThreads), 0, st, 
                 in, f.vals, f.info + kInfoM, 0u, 8 * p, hist, status, s.counters + 5 + p, f.info, 0xFFFFFFFFu,
-                nullptr, nullptr));
+                nullptr, nullptr, nullptr));
         else
             CK(launch_pdl(k_radix_pass<false, false>, dim3((unsigned)bc), dim3(kSortThreads), 0, st, 
                 in, (p % 2 == 0) ? s.items_b : s.items_a, f.info + kInfoM, 0u, 8 * p, hist, status,
-                s.counters + 5 + p, f.info, 0xFFFFFFFFu, nullptr, nullptr));
+                s.counters + 5 + p, f.info, 0xFFFFFFFFu, nullptr, nullptr, nullptr));
         count_launches();
         CK(cudaGetLastError());
     }
