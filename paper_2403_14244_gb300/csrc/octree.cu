@@ -13,7 +13,8 @@
 // order whose split (adding its non-empty children minus one) does not fit.
 // The prefix is found by a radix selection on the 64-bit key (8 bits at a time,
 // histograms weighted by the leaves each split adds), and then on the id among
-// equal keys, by one cluster of CTAs that holds every key in shared memory. The
+// equal keys, by one cluster of CTAs that holds every key in shared memory (or by one
+// CTA: few cells, or a device or partition of one that does not hold the cluster). The
 // leaves are then emitted in id order, a CTA per chunk of cells placed after the
 // leaves of the chunks before it. (2M points, seven levels, a budget of 500K: 752 us
 // before, 478 with all that follows here, of which the kernels 286.)
@@ -206,10 +207,18 @@ constexpr int kSelCtas = 16, kSelThreads = 1024;
 constexpr long long kSelShare = (299593 + kSelCtas - 1) / kSelCtas;  // cells of levels 0 .. 6 (L <= 7)
 constexpr int kSelSpan = (int)((kSelShare + kSelThreads / 32 - 1) / (kSelThreads / 32));  // cells per warp
 constexpr size_t kSelSmem = (size_t)kSelShare * 9 + 1 + (size_t)kSelSpan * (kSelThreads / 32) * 2;
+// Up to this many levels (4681 cells above the finest) one CTA is the better form: 20,000 points on
+// 4 and 5 levels take 145 and 172 us in all, 174 and 192 with the cluster; on 6 and 7 levels 315 and 1437
+// against 218 and 262, which is what a device without room for the cluster takes.
+constexpr int kSelOneLevels = 5;
 static_assert(kSelShare <= 65536 && kSelShare % 2 == 1, "16-bit lists, placed after the odd bytes of the increments");
 static_assert(kSelSmem + 4096 <= 227 * 1024, "shared memory of a CTA");
+//
+// Without CLUSTER, one CTA does it all: the keys are formed in place of the errors, a level
+// after another, and a pass goes over every cell in global memory.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kSelThreads) k_oct_select(const uint32_t* __restrict__ cnt,
-                                                            const unsigned long long* __restrict__ err,
+                                                            unsigned long long* __restrict__ err,
                                                             const uint8_t* __restrict__ inc8, long long items,
                                                             long long k_max, uint8_t* __restrict__ split) {
     extern __shared__ unsigned long long s_key[];                       // [kSelShare]
@@ -219,14 +228,23 @@ __global__ void __launch_bounds__(kSelThreads) k_oct_select(const uint32_t* __re
     __shared__ OctSel s;
     __shared__ int s_b;
     namespace cg = cooperative_groups;
-    const cg::cluster_group cluster = cg::this_cluster();
+    const cg::cluster_group cluster = cg::this_cluster();  // (of one CTA, without CLUSTER)
     const int t = threadIdx.x, lane = t & 31;
-    const long long first = (long long)cluster.block_rank() * kSelShare;
-    const int mine = (int)max(0ll, min(kSelShare, items - first));
+    const long long first = CLUSTER ? (long long)cluster.block_rank() * kSelShare : 0;
+    const int mine = CLUSTER ? (int)max(0ll, min(kSelShare, items - first)) : (int)items;
+    auto key_of = [&](int i) { return CLUSTER ? s_key[i] : err[i]; };
+    auto inc_of = [&](int i) { return (uint32_t)(CLUSTER ? s_inc[i] : inc8[i]); };
     const int w0 = (t >> 5) * kSelSpan, w1 = min(mine, w0 + kSelSpan);  // this warp's cells
     uint16_t* list = s_list + w0;
     int left = 0;  // its candidates: cells whose split adds leaves, and whose key the digits so far allow
-    for (int i0 = w0; i0 < w1; i0 += 32) {
+    if constexpr (!CLUSTER) {
+        for (int l = 1; oct_off(l) < items; ++l) {  // (the parents' keys are complete)
+            for (long long m = t; m < (1ll << (3 * l)); m += kSelThreads)
+                err[oct_off(l) + m] = min(err[oct_off(l) + m], err[oct_off(l - 1) + (m >> 3)]);
+            __syncthreads();
+        }
+    }
+    for (int i0 = CLUSTER ? w0 : w1; i0 < w1; i0 += 32) {
         const int i = i0 + lane;
         bool cand = false;
         if (i < w1) {
@@ -257,19 +275,21 @@ __global__ void __launch_bounds__(kSelThreads) k_oct_select(const uint32_t* __re
         const int sh = 8 * (key ? 7 - pass : 10 - pass);
         const unsigned long long hi = key && pass == 0 ? 0ull : (~0ull << (sh + 8));
         int kept = 0;
-        for (int j0 = 0; j0 < left; j0 += 32) {
+        // the warp's list, or every 32nd run of 32 cells
+        for (int j0 = CLUSTER ? 0 : t & ~31; j0 < (CLUSTER ? left : mine); j0 += CLUSTER ? 32 : kSelThreads) {
             uint32_t c = 0, d = 0;
             int i = 0;
-            if (j0 + lane < left) {
-                i = list[j0 + lane];
-                const unsigned long long k = s_key[i], id = (unsigned long long)(first + i);
+            if (j0 + lane < (CLUSTER ? left : mine)) {
+                i = CLUSTER ? list[j0 + lane] : j0 + lane;
+                const unsigned long long k = key_of(i), id = (unsigned long long)(first + i);
                 const bool in = key ? (k & hi) == prefix : k == prefix && (id & hi) == idp;
                 d = (uint32_t)((key ? k : id) >> sh) & 0xFFu;
-                if (in) c = s_inc[i];
+                if (in) c = inc_of(i);
+                if (!CLUSTER && c == 0xFFu) c = 0;
             }
             uint32_t on = __ballot_sync(0xffffffffu, c != 0);
             // the list shrinks in place: what is written lies at or below what every lane has read
-            if (c) list[kept + __popc(on & ((1u << lane) - 1u))] = (uint16_t)i;
+            if (CLUSTER && c) list[kept + __popc(on & ((1u << lane) - 1u))] = (uint16_t)i;
             kept += __popc(on);
             // the errors' top digits (sign and exponent) are few: a digit that many lanes share is added once
 #pragma unroll
@@ -284,14 +304,20 @@ __global__ void __launch_bounds__(kSelThreads) k_oct_select(const uint32_t* __re
             if (c) atomicAdd(&s_h[d], c);
         }
         left = kept;
-        cluster.sync();  // every CTA's histogram is complete
-        if (t < 256) {
-            uint32_t h = 0;  // (all increments together are below 7 x 299593)
+        if constexpr (CLUSTER) {
+            cluster.sync();  // every CTA's histogram is complete
+            if (t < 256) {
+                uint32_t h = 0;  // (all increments together are below 7 x 299593)
 #pragma unroll
-            for (int r = 0; r < kSelCtas; ++r) h += cluster.map_shared_rank(s_h, r)[t];
-            s_tot[t] = h;
+                for (int r = 0; r < kSelCtas; ++r) h += cluster.map_shared_rank(s_h, r)[t];
+                s_tot[t] = h;
+            }
+            cluster.sync();  // no CTA reads another's histogram any more
+        } else {
+            __syncthreads();
+            if (t < 256) s_tot[t] = s_h[t];
+            __syncthreads();
         }
-        cluster.sync();  // no CTA reads another's histogram any more
         // thread t < 256 holds one bin (bin 255 - t for the key, taken from the top; bin t for the id); an
         // inclusive scan gives each the increments at and above it (key) or at and below it (id)
         const int bin = key ? 255 - t : t;
@@ -353,7 +379,8 @@ __global__ void __launch_bounds__(kSelThreads) k_oct_select(const uint32_t* __re
     for (int i = t; i < mine; i += kSelThreads) {
         const long long id = first + i;
         bool sp = false;
-        if (root && s_inc[i] != 0xFFu) sp = s.all != 0 || s_key[i] > s.prefix || (s_key[i] == s.prefix && id <= s.ihi);
+        if (root && inc_of(i) != 0xFFu)
+            sp = s.all != 0 || key_of(i) > s.prefix || (key_of(i) == s.prefix && id <= s.ihi);
         split[id] = sp ? 1 : 0;
     }
 }
@@ -523,22 +550,28 @@ size_t octree_work_bytes(int L) {
     return oct_work(L, nullptr).bytes;
 }
 
-// The selection's cluster: its shared memory and its size (above the portable eight) opted into, once per device.
-static cudaError_t sel_opt_in() {
+// Whether the device holds the selection's cluster (with what the current context has of it): its
+// shared memory and its size (above the portable eight) are opted into, once per device.
+static bool sel_cluster_fits(const cudaLaunchConfig_t& cfg) {
     static std::mutex mu;
     static bool done[128] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 128) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return cudaSuccess;
-    if ((e = cudaFuncSetAttribute(k_oct_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_oct_select, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-        return e;
-    done[dev] = true;
-    return cudaSuccess;
+    int dev = 0, clusters = 0;
+    auto ok = [](cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();  // (the other form needs neither)
+        return e == cudaSuccess;
+    };
+    if (!ok(cudaGetDevice(&dev)) || dev < 0 || dev >= 128) return false;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!done[dev]) {
+            if (!ok(cudaFuncSetAttribute(k_oct_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSelSmem)) ||
+                !ok(cudaFuncSetAttribute(k_oct_select<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
+                return false;
+            done[dev] = true;
+        }
+    }
+    return ok(cudaOccupancyMaxActiveClusters(&clusters, k_oct_select<true>, &cfg)) && clusters > 0;
 }
 
 cudaError_t launch_octree_init(const float* pts, const float* cols, long long npts, const float lo[3], float side,
@@ -581,7 +614,6 @@ cudaError_t launch_octree_init(const float* pts, const float* cols, long long np
         k_oct_err<<<(unsigned)ceil_div(items, 256), 256, 0, st>>>(o.cnt, o.sums, items, o.err, o.inc8);
         launches += 2;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = sel_opt_in()) != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kSelCtas);
         cfg.blockDim = dim3(kSelThreads);
@@ -593,8 +625,13 @@ cudaError_t launch_octree_init(const float* pts, const float* cols, long long np
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, k_oct_select, (const uint32_t*)o.cnt, (const unsigned long long*)o.err,
-                               (const uint8_t*)o.inc8, items, k_max, o.split);
+        if (L > kSelOneLevels && sel_cluster_fits(cfg))
+            e = cudaLaunchKernelEx(&cfg, k_oct_select<true>, (const uint32_t*)o.cnt, o.err, (const uint8_t*)o.inc8,
+                                   items, k_max, o.split);
+        else {
+            k_oct_select<false><<<1, kSelThreads, 0, st>>>(o.cnt, o.err, o.inc8, items, k_max, o.split);
+            e = cudaGetLastError();
+        }
         ++launches;
         if (e != cudaSuccess) return e;
     }
