@@ -284,9 +284,9 @@ __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_sub(
 
 // The backward over walk segments: one-warp CTAs, all resident, take work from
 // one counter: first the segments the forward closed, then each block's last
-// segment (its whole walk when it closed none). Every piece walks at most
-// seg.stride list positions (unless the pool ran out), so no block's long walk
-// sets the kernel's length.
+// segment (its whole walk when it closed none). A piece walks at most 1024
+// list positions, or 256 (SegLayout), unless the pool ran out, so no block's long
+// walk sets the kernel's length.
 template <int TS>
 __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_segs(const uint2* __restrict__ ranges,
                                                            const uint32_t* __restrict__ vals,
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_segs(const uint2*
             block = it.x;
             lo = it.y;
             hi = it.z;
-            slot = it.w;
+            slot = u;
         } else {
             block = u - items;
             const uint4 l = seg.last[block];

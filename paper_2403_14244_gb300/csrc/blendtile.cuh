@@ -197,7 +197,6 @@ __device__ __forceinline__ void stage_begin(Stager& S, uint32_t total, uint32_t 
 struct FwdQueue {
     FwdEntry e[kQueue];
     Stager st;
-    uint32_t slots[kSegMaxPerBlock];  // pool slots of the segments closed (with walk segments)
 };
 
 __device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -328,8 +327,10 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
 #pragma unroll
     for (int i = 0; i < 2; ++i) s.C[i][0] = s.C[i][1] = s.C[i][2] = s.D[i][0] = s.D[i][1] = s.D[i][2] = 0.f;
     s.last[0] = s.last[1] = 0;
-    // segment state (warp-uniform): where the open segment starts (the last cut), the segments closed
-    uint32_t seg_lo = 0, seg_n = 0;
+    // segment state (warp-uniform): where the open segment starts, the segments closed, the last one's slot,
+    // and the list positions between cuts
+    uint32_t seg_lo = 0, seg_n = 0, seg_last = kSegNone;
+    uint32_t stride = seg.stride;
     bool seg_stop = false;
     uint32_t reserved = kSegNone;  // lane 0: the pool slot taken for the next close (its atomic is in flight meanwhile)
     const bool segs = SEG && seg.slots != 0;
@@ -353,31 +354,30 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
     for (uint32_t b = 0; b * 32 < n && !done; ++b) {
         const uint32_t b0 = b * 32;
         if constexpr (SEG) {
-            if (segs && b0 > 0 && (b0 & (seg.stride - 1)) == 0) {
+            if (segs && b0 > 0 && (b0 & (stride - 1)) == 0) {
                 if (queued && walk(queued)) break;
                 // close the open segment here if it holds blends: each pixel's T is that after every
                 // entry before b0, and the segment's own colour is kept until the walk has ended and
                 // the colour behind the cut can be summed
                 const uint32_t hi = __reduce_max_sync(0xffffffffu, max(s.last[0], s.last[1]));
-                if (hi > seg_lo && !seg_stop && seg_n < kSegMaxPerBlock) {
-                    uint32_t pool_slot = 0;
+                if (hi <= seg_lo) {
+                    seg_lo = b0;  // nothing blended since the last cut
+                } else if (!seg_stop) {
+                    uint32_t pool_slot = kSegNone;
                     if (lane == 0) {
-                        if (reserved == kSegNone) {  // first close: this slot and the next one
-                            pool_slot = atomicAdd(&seg.ctrl->slots_used, 2u);
-                            reserved = pool_slot + 1;
-                        } else {
+                        if (reserved == kSegNone) reserved = atomicAdd(&seg.ctrl->slots_used, 1u);
+                        if (reserved < seg.fine || (b0 & (kSegStride - 1)) == 0) {
                             pool_slot = reserved;
-                            reserved = atomicAdd(&seg.ctrl->slots_used, 1u);
+                            if (pool_slot < seg.slots) reserved = atomicAdd(&seg.ctrl->slots_used, 1u);
                         }
                     }
                     pool_slot = __shfl_sync(0xffffffffu, pool_slot, 0);
-                    if (pool_slot >= seg.slots) {
+                    if (pool_slot == kSegNone) {
+                        stride = kSegStride;  // the slots left are for longer pieces
+                    } else if (pool_slot >= seg.slots) {
                         seg_stop = true;  // pool full: the block's last segment takes the rest
                     } else {
-                        if (lane == 0) {
-                            seg.items[pool_slot] = make_uint4(block, seg_lo, hi, pool_slot);
-                            Q.slots[seg_n] = pool_slot;
-                        }
+                        if (lane == 0) seg.items[pool_slot] = make_uint4(block, seg_lo, hi, seg_last);
                         const float(&own)[2][3] = seg_n == 0 ? s.C : s.D;  // the first segment's colour is all there is
                         float4* st = seg.state(pool_slot) + lane;
                         st[0] = make_float4(s.T.x, own[0][0], own[0][1], own[0][2]);
@@ -385,6 +385,7 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
 #pragma unroll
                         for (int i = 0; i < 2; ++i) s.D[i][0] = s.D[i][1] = s.D[i][2] = 0.f;
                         ++seg_n;
+                        seg_last = pool_slot;
                         seg_lo = b0;
                     }
                 }
@@ -414,9 +415,7 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
         if (segs) {
             const uint32_t hi = __reduce_max_sync(0xffffffffu, max(s.last[0], s.last[1]));
             if (lane == 0) {
-                // (no segment closed: the last segment is the whole walk; lo = kSegNone: no blend after the last cut)
-                seg.last[block] = seg_n == 0 ? make_uint4(0u, 0u, kSegNone, 0u)
-                                             : make_uint4(seg_n, hi > seg_lo ? seg_lo : kSegNone, hi, 0u);
+                seg.last[block] = make_uint4(seg_n, hi > seg_lo ? seg_lo : kSegNone, hi, 0u);
                 if (reserved != kSegNone && reserved < seg.slots)
                     seg.items[reserved] = make_uint4(kSegNone, 0u, 0u, kSegNone);  // taken, not used
             }
@@ -431,8 +430,9 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
                     for (int ch = 0; ch < 3; ++ch) S[h][ch] = fmaf(h ? s.T.y : s.T.x, bg[ch], s.D[h][ch]);
-                for (uint32_t i = seg_n; i-- > 0;) {
-                    float4* st = seg.state(Q.slots[i]) + lane;
+                for (uint32_t slot_i = seg_last; slot_i != kSegNone;) {
+                    float4* st = seg.state(slot_i) + lane;
+                    const uint32_t before = lane == 0 ? seg.items[slot_i].w : 0u;  // (lane 0 wrote it)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const float4 v = st[32 * h];
@@ -441,6 +441,7 @@ __device__ __forceinline__ void blend_block_fwd(int bx, int by, int width, int h
                         S[h][1] += v.z;
                         S[h][2] += v.w;
                     }
+                    slot_i = __shfl_sync(0xffffffffu, before, 0);
                 }
             }
         }

@@ -388,22 +388,28 @@ size_t sort_scratch_bytes(int64_t n, int64_t capacity, int64_t tiles_x, int64_t 
 // blends: it saves each pixel's state there (T, and the colour composited
 // behind that position, once the walk has ended) in a pool slot, so that the
 // backward can walk every segment in parallel instead of one block walking its
-// whole list. A closed segment is items[slot] = (block, lo, hi, slot): list
-// positions relative to the tile's first entry, lo = the cut it starts at, hi =
+// whole list. A closed segment is items[slot] = (block, lo, hi, the slot of the
+// block's segment before it or kSegNone): list positions relative to the tile's
+// first entry, lo = the last cut before its first blend, hi =
 // one past its last blend, the state at hi in slot's pixels; a slot taken but not
 // used holds block = kSegNone. A block's last segment, which ends with the final
 // state (T_final and the background), is last[block] = (segments closed, lo,
-// hi, -); lo = kSegNone when it holds no blend. The pieces live in scratch that
+// hi, -); lo = kSegNone when it holds no blend. A segment spans at most a stride
+// (kSegStride once the slots for a shorter one are taken), unless the pool is full: the
+// block's last segment then takes the rest. The pieces live in scratch that
 // binning no longer needs once the entries are placed: the depth-sort item
 // buffers and the level-1 counts.
 constexpr uint32_t kSegNone = 0xFFFFFFFFu;
-constexpr int kSegMaxPerBlock = 64;          // segments a block closes at most (the rest stay in its last one)
 // List positions between cuts, multiples of the blends' 32-entry batches. A frame of few blocks leaves
 // most of the backward's warps without work, and its time is that of the longest piece: with cuts every
 // 256 positions instead of 1024, the training step of 30,000 Gaussians at 401 x 299 pixels (1976 blocks,
 // walks up to 870) takes 147 us instead of 175 (512: 172). With many blocks the cuts gain the backward
 // about 1 % (3M training step 1340 -> 1326 us) and cost a forward without a backward up to 4 % (200,000
-// Gaussians at 1001 x 667, 10584 blocks: 190 -> 199 us), so those keep 1024.
+// Gaussians at 1001 x 667, 10584 blocks: 190 -> 199 us), so those keep 1024. Of the pool, half of its
+// first part is kept for cuts at multiples of 1024: with a pool that the shorter pieces may use up, the
+// blocks that walk on after that set the backward's time (20,000 faint Gaussians at 64 x 48 pixels, lists up to
+// 10,000: 585 us, 355 with the half kept; 200,000 at 128 x 96: 220 and 73; kept though not needed, 166,600
+// at 215 x 144: 58 and 70).
 constexpr uint32_t kSegStride = 1024, kSegStrideFew = 256;
 constexpr int64_t kSegFewBlocks = 8192;
 struct SegCtrl {                             // all zeroed before each forward; next (the
@@ -412,13 +418,14 @@ struct SegCtrl {                             // all zeroed before each forward; 
 struct SegLayout {
     SegCtrl* ctrl;
     uint4* last;      // [blocks] (closed, lo, hi, -) of each block's last segment
-    uint4* items;     // [slots] (block, lo, hi, slot) of each closed segment
+    uint4* items;     // [slots] (block, lo, hi, slot before) of each closed segment
     float4* pool;     // [slots][64] (T, S_r, S_g, S_b) per pixel of the block, pixel = row * 8 + column:
     float4* pool2;    // slots below `split` in pool, the others in pool2
     uint32_t split;
     uint32_t slots;   // 0: segments off
     uint32_t blocks;
-    uint32_t stride;  // a power of two
+    uint32_t stride;  // list positions between cuts, kSegStride or fewer,
+    uint32_t fine;    // fewer while slots below this are left
     __device__ __forceinline__ float4* state(uint32_t slot) const {
         return slot < split ? pool + (size_t)slot * 64 : pool2 + (size_t)(slot - split) * 64;
     }
@@ -445,6 +452,7 @@ __host__ __device__ inline SegLayout seg_layout(void* base, size_t bytes, void* 
     L.slots = (uint32_t)(slots + (int64_t)more);
     L.blocks = (uint32_t)blocks;
     L.stride = blocks <= kSegFewBlocks ? kSegStrideFew : kSegStride;
+    L.fine = L.slots - L.split / 2;
     return L;
 }
 int64_t sort_walk_chunks(int64_t tiles_x, int64_t tiles_y);
