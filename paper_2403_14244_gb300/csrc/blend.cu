@@ -67,6 +67,11 @@ __device__ __forceinline__ float fast_rcp(float x) {
     return y;
 }
 
+// (A pixel that did not blend an entry multiplies its T by fast_rcp(1), thousands of times
+// in a long walk. That this is 1 exactly is not promised by the instruction's error bound
+// of one ulp; it holds on this hardware, and a test holds it: selects for T cost 1 % of the
+// backward, 299 us a 1080p view of 1M Gaussians without and 302 with.)
+//
 // The adjoint of one entry at the warp's 64 pixels, summed over the warp: lane
 // 4 v holds term v of (dalpha g (dx, dy, d^2, 1), dr, dg, db, -). With FINITE
 // (every G of the warp and every distance is finite), a pixel that did not blend
