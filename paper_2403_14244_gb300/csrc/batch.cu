@@ -42,7 +42,7 @@ struct Fanout {
 
 // Every view of the batch for one Gaussian per thread: the Gaussian's mean,
 // scale, opacity and colour row are read once and projected for each view in
-// turn (what project_one writes into that view's frame), the view table staged
+// turn (what project_one_vals writes into that view's frame), the view table staged
 // kViewChunk entries at a time in shared memory. The scene is read once per
 // batch, not once per view; the per-view writes stay coalesced across a warp.
 constexpr int kViewChunk = 16;

@@ -294,15 +294,5 @@ __device__ __forceinline__ void project_one_with(const float4* __restrict__ ms, 
     project_one_vals<DEG>(__ldg(ms + i), __ldg(op + i), load_c, P, rec, rect, disc, count, depth_key);
 }
 
-template <int DEG>
-__device__ __forceinline__ void project_one(const float4* __restrict__ ms, const float* __restrict__ op,
-                                            const float* __restrict__ col, int64_t i, const ViewParams& P,
-                                            float4* __restrict__ rec, uint2* __restrict__ rect,
-                                            float4* __restrict__ disc, uint32_t* __restrict__ count,
-                                            uint32_t* __restrict__ depth_key) {
-    project_one_with<DEG>(ms, op, [&](float c[48]) { load_color<DEG>(col, i, c); }, i, P, rec, rect, disc, count,
-                          depth_key);
-}
-
 }  // namespace
 }  // namespace igs
