@@ -150,20 +150,18 @@ __global__ void __launch_bounds__(TS* TS) k_blend_persistent(const BatchView* __
 }
 
 // Sub-tile blend: one warp per 8 x 8 pixel block of every view's binning tiles
-// (block w of the batch: tile w / (TS/8)^2, block w % (TS/8)^2 of it), walking the
+// (CTA b of the batch: tile b / (TS/8)^2, block b % (TS/8)^2 of it), walking the
 // tile's entries as the one-view blend does; each block stops on its own. The
 // hardware block scheduler balances the mixed view sizes, so the launch is not
 // persistent.
-constexpr int kSubWarps = 1;  // warps (8 x 8 blocks) per CTA
 template <int TS>
-__global__ void __launch_bounds__(32 * kSubWarps, 28 / kSubWarps) k_blend_batch_sub(const BatchView* __restrict__ views, int V,
-                                                                        uint32_t tiles_total, BlendParams P,
-                                                                        float* __restrict__ images,
-                                                                        uint32_t* __restrict__ work) {
+__global__ void __launch_bounds__(32, kFwdMinCtas) k_blend_batch_sub(const BatchView* __restrict__ views, int V,
+                                                                     uint32_t tiles_total, BlendParams P,
+                                                                     float* __restrict__ images,
+                                                                     uint32_t* __restrict__ work) {
     constexpr uint32_t SUB = TS / 8, NS = SUB * SUB;
-    __shared__ FwdQueue s_q[kSubWarps];
-    const uint32_t b = blockIdx.x * kSubWarps + (threadIdx.x >> 5);
-    const uint32_t w = b / NS, q = b % NS;
+    __shared__ FwdQueue s_q;
+    const uint32_t w = blockIdx.x / NS, q = blockIdx.x % NS;
     if (w >= tiles_total) return;
     const BatchView& bv = views[view_of(views, V, w)];
     if (bv.info[kInfoAbort]) return;
@@ -172,7 +170,7 @@ __global__ void __launch_bounds__(32 * kSubWarps, 28 / kSubWarps) k_blend_batch_
     const uint32_t tx = t % (uint32_t)vp.tiles_x, ty = t / (uint32_t)vp.tiles_x;
     blend_block_fwd<false>((int)((tx * SUB + q % SUB) * 8), (int)((ty * SUB + q / SUB) * 8), vp.width, vp.height,
                            bv.ranges[t], bv.vals, bv.rec, P.alpha_min, P.alpha_max, P.t_min, P.bg,
-                           s_q[threadIdx.x >> 5], images + bv.img_off, nullptr, nullptr);
+                           s_q, images + bv.img_off, nullptr, nullptr);
 }
 
 template <int TS, int B>
@@ -317,13 +315,13 @@ cudaError_t launch_render_batch(const igs_batch& b, const igs_frame* frames, con
     bool sub = false;
     if (!blend_variant(b.tile, b.blend_batch, &fn, &sub)) return cudaErrorInvalidValue;
     const int64_t per_tile = sub ? (int64_t)(b.tile / 8) * (b.tile / 8) : 1;
-    const unsigned nblocks = (unsigned)(sub ? std::max<int64_t>(1, ceil_div(b.tiles_total * per_tile, kSubWarps))
+    const unsigned nblocks = (unsigned)(sub ? std::max<int64_t>(1, b.tiles_total * per_tile)
                                             : std::max<int64_t>(1, std::min<int64_t>(b.persistent_blocks, b.tiles_total)));
     uint32_t tt = (uint32_t)b.tiles_total;
     int Vi = V;
     BlendParams bpp = bp;
     void* args[] = {(void*)&table, (void*)&Vi, (void*)&tt, (void*)&bpp, (void*)&images, (void*)&work};
-    CK(cudaLaunchKernel(fn, dim3(nblocks), dim3(sub ? 32 * kSubWarps : b.tile * b.tile), args, 0, st));
+    CK(cudaLaunchKernel(fn, dim3(nblocks), dim3(sub ? 32 : b.tile * b.tile), args, 0, st));
     count_launches();
 #undef CK
     return cudaSuccess;

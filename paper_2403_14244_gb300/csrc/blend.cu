@@ -18,10 +18,6 @@
 namespace igs {
 namespace {
 
-// Warps (8 x 8 blocks) per CTA of the forward, and resident CTAs per SM asked of the compiler.
-constexpr int kFwdWarps = 1;
-constexpr int kFwdMinCtas = 28;
-
 // Zeros to n4 float4 at p (none if p is null), spread over the grid: the
 // forward blend of a training step clears the 2D gradient for the adjoint that
 // follows. The blend is bound by instruction issue and leaves HBM mostly idle,
@@ -246,32 +242,31 @@ __device__ __forceinline__ void blend_block_bwd(int bx, int by, uint2 rg, const 
 // Per pixel the walk, the arithmetic and the result are those of the whole-tile
 // kernels.
 template <int TS>
-__global__ void __launch_bounds__(32 * kFwdWarps, kFwdMinCtas) k_blend_fwd_sub(
+__global__ void __launch_bounds__(32, kFwdMinCtas) k_blend_fwd_sub(
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ rec, BlendParams P,
     float* __restrict__ img, float* __restrict__ T_final, uint32_t* __restrict__ n_contrib,
     const uint32_t* __restrict__ info, SegLayout seg, const uint32_t* __restrict__ tile_order,
     float4* __restrict__ clear, uint64_t clear4) {
     pdl_wait();
     constexpr int SUB = TS / 8;
-    __shared__ FwdQueue s_q[kFwdWarps];
+    __shared__ FwdQueue s_q;
     clear_slice(clear, clear4);
     if (info[kInfoAbort]) return;
-    const uint32_t at = blockIdx.x * kFwdWarps + (threadIdx.x >> 5);  // in starting order
-    const int q = (int)(at % (SUB * SUB));
+    const int q = (int)(blockIdx.x % (SUB * SUB));
     const uint32_t tiles = (uint32_t)(P.tiles_x * P.tiles_y);
-    uint32_t t = at / (SUB * SUB);
-    if (t >= tiles) return;
+    uint32_t t = blockIdx.x / (SUB * SUB);  // in starting order
     if (tile_order && (t = tile_order[t]) >= tiles) return;  // (a frame whose binning never ordered its tiles)
     const int tile = (int)t;
     const int tx = tile % P.tiles_x, ty = tile / P.tiles_x;
     blend_block_fwd<TS != 8>((tx * SUB + q % SUB) * 8, (ty * SUB + q / SUB) * 8, P.width, P.height, ranges[tile], vals,
-                             rec, P.alpha_min, P.alpha_max, P.t_min, P.bg, s_q[threadIdx.x >> 5], img, T_final,
+                             rec, P.alpha_min, P.alpha_max, P.t_min, P.bg, s_q, img, T_final,
                              n_contrib, seg, (uint32_t)(tile * SUB * SUB + q));
 }
 
 // The backward of a block's whole walk (8-pixel tiles; larger ones when the
 // frame has no room for walk segments).
 constexpr int kBwdMinCtas = 24;  // resident one-warp CTAs per SM asked of the compiler
+static_assert(kBwdMinCtas * (sizeof(BwdQueue) + 1024) <= 228 * 1024, "resident CTAs per SM");
 template <int TS>
 __global__ void __launch_bounds__(32, kBwdMinCtas) k_blend_bwd_sub(
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ rec, BlendParams P,
@@ -370,7 +365,7 @@ cudaError_t launch_blend_fwd(const igs_frame& f, const BlendParams& bp, float* i
     }
     const uint32_t* tile_order = f.n > 0 ? sort_scratch(f).tile_order : nullptr;  // (an empty scene bins nothing)
     const int64_t sub = f.tile / 8;
-    const dim3 grid((unsigned)ceil_div((int64_t)tiles * sub * sub, kFwdWarps)), block(32 * kFwdWarps);
+    const dim3 grid((unsigned)((int64_t)tiles * sub * sub)), block(32);
     switch (f.tile) {
         case 8: e = launch_pdl(k_blend_fwd_sub<8>, grid, block, 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, tile_order, clear, clear4); break;
         case 16: e = launch_pdl(k_blend_fwd_sub<16>, grid, block, 0, st, rg, f.vals, rec, bp, img, f.T_final, f.n_contrib, f.info, seg, tile_order, clear, clear4); break;

@@ -198,6 +198,10 @@ struct FwdQueue {
     FwdEntry e[kQueue];
     Stager st;
 };
+// Resident one-warp CTAs per SM asked of the compiler (72 registers a thread; 27 and 28 take the same
+// time), as many as an SM's 228 KB of shared memory holds, 1 KB of it the system's for each.
+constexpr int kFwdMinCtas = 28;
+static_assert(kFwdMinCtas * (sizeof(FwdQueue) + 1024) <= 228 * 1024, "resident CTAs per SM");
 
 __device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 pk_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
