@@ -342,6 +342,22 @@ __global__ void __launch_bounds__(kTileScanThreads) k_tile_scan(const int32_t* g
     }
 }
 
+// Inclusive prefix of n words in shared memory, `step` apart, by one thread: eight reads in
+// flight (one by one, each waited for the write before it).
+__device__ __forceinline__ void prefix_in_place(int32_t* p, int step, int n) {
+    int32_t run = 0;
+    for (int i = 0; i < n; i += 8) {
+        int32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = i + k < n ? p[(i + k) * step] : 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            run += v[k];
+            if (i + k < n) p[(i + k) * step] = run;
+        }
+    }
+}
+
 // One block, grid in shared memory (cells <= kGridSmemCells): the row prefix of
 // the difference grid, the tile ranges, the tile-digit histograms, every digit
 // histogram (4 depth + `passes` tile rows) turned into exclusive offsets, and
@@ -377,16 +393,10 @@ __global__ void __launch_bounds__(kTilesSmallThreads) k_tiles_small(const int32_
         if (tid == 0) info[kInfoSkipTop] = (nz <= 1u && ld_cg(info + kInfoKeyWrap) == 0u) ? 1u : 0u;
     }
     if (diff2d) {  // rectangles were added as 2D differences: a prefix down each column first
-        for (int x = tid; x < tiles_x; x += blockDim.x) {
-            int32_t run = 0;
-            for (int y = 0; y < tiles_y; ++y) { run += s_g[y * gx + x]; s_g[y * gx + x] = run; }
-        }
+        for (int x = tid; x < tiles_x; x += blockDim.x) prefix_in_place(s_g + x, gx, tiles_y);
         __syncthreads();
     }
-    for (int y = tid; y < tiles_y; y += blockDim.x) {
-        int32_t run = 0;
-        for (int x = 0; x < tiles_x; ++x) { run += s_g[y * gx + x]; s_g[y * gx + x] = run; }
-    }
+    for (int y = tid; y < tiles_y; y += blockDim.x) prefix_in_place(s_g + y * gx, 1, tiles_x);
     __syncthreads();
     const uint32_t tiles = (uint32_t)tiles_x * tiles_y;
     const uint32_t per = (tiles + kTilesSmallThreads - 1) / kTilesSmallThreads;
