@@ -567,7 +567,7 @@ IGS_API void igs_debug_silence_lookback_once(void);
 /* Walk segments (observability; the paper has no counterpart). With 16- and
  * 32-pixel tiles the forward blend (igs_render_fwd) cuts the walk of an 8 x 8
  * pixel block through its tile's entries every 256 (up to 8192
- * blocks) or 1024 list positions where the
+ * blocks, while room for short segments lasts) or 1024 list positions where the
  * block has blended since the previous cut, and saves the pixels' state there,
  * so that igs_blend_bwd walks the pieces in parallel (Eq. 4's adjoint is the same;
  * only the order of the additions changes). Writes to *host_count the pool slots

@@ -405,7 +405,9 @@ constexpr uint32_t kSegNone = 0xFFFFFFFFu;
 // 256 positions instead of 1024, the training step of 30,000 Gaussians at 401 x 299 pixels (1976 blocks,
 // walks up to 870) takes 147 us instead of 175 (512: 172). With many blocks the cuts gain the backward
 // about 1 % (3M training step 1340 -> 1326 us) and cost a forward without a backward up to 4 % (200,000
-// Gaussians at 1001 x 667, 10584 blocks: 190 -> 199 us), so those keep 1024. Of the pool, half of its
+// Gaussians at 1001 x 667, 10584 blocks: 190 -> 199 us), so those keep 1024. With few blocks they cost the
+// forward blend 0 to 18 % (20,000 Gaussians at 320 x 240: 20 -> 23 us; 11,600 at 436 x 332: 14.6 -> 17.2;
+// 100,000 at 640 x 480: 36 -> 37) and gain the backward 72 -> 42, 44 -> 37 and 85 -> 79 there. Of the pool, half of its
 // first part is kept for cuts at multiples of 1024: with a pool that the shorter pieces may use up, the
 // blocks that walk on after that set the backward's time (20,000 faint Gaussians at 64 x 48 pixels, lists up to
 // 10,000: 585 us, 355 with the half kept; 200,000 at 128 x 96: 220 and 73; kept though not needed, 166,600

@@ -1,7 +1,7 @@
 """Where the forward blend cuts a block's walk for the backward: list lengths around the stride of
-frames of few blocks (256) and where it doubles, lists longer than 64 segments of it, blocks whose
-first blends lie far down the list, and both sides of the number of blocks (8192) from which the
-stride is 1024. Gradients against the oracle, or, in the larger images, against 8-pixel tiles,
+frames of few blocks (256), lists of more than 64 segments of it and of more than the room for short
+segments, blocks whose first blends lie far down the list, and both sides of the number of blocks
+(8192) from which the stride is 1024. Gradients against the oracle, or, in the larger images, against 8-pixel tiles,
 whose walks are not cut."""
 import numpy as np
 import pytest
