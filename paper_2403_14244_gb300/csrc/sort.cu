@@ -585,7 +585,6 @@ struct DiscRef {
     int tile;
     float inv_tile;
     int footprint;
-    int tiles_x;
 };
 
 using Placer1 = Placer<u64, kStage1>;      // level 1: (column span << 32 | Gaussian id) items
@@ -619,7 +618,9 @@ __device__ __forceinline__ void diff_to_counts(const uint32_t* d, uint32_t B, in
 // that of order[p]) so that the placement reads them without a gather.
 template <bool DISCS>
 __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* __restrict__ order,
-                                                                DiscRef disc, uint32_t rows,
+                                                                const uint2* __restrict__ rect,
+                                                                const float4* __restrict__ discs, int tile,
+                                                                float inv_tile, uint32_t tiles_x, uint32_t rows,
                                                                 uint32_t cmax, uint32_t* __restrict__ H1,
                                                                 uint2* __restrict__ srect,
                                                                 const uint32_t* __restrict__ info) {
@@ -645,8 +646,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_rows_count(const uint32_t* 
             for (int k = 0; k < kWalkUnroll; ++k) {
                 uint2 r = make_uint2(1u << 16, 0u);  // rows 1..0: none
                 if (g[k] != 0xFFFFFFFFu) {
-                    r = disc.rect[g[k]];
-                    if (DISCS) r = touched_rows(r, disc.disc + g[k], disc.tile, disc.inv_tile, disc.tiles_x);
+                    r = rect[g[k]];
+                    if (DISCS) r = touched_rows(r, discs + g[k], tile, inv_tile, (int)tiles_x);
                 }
                 ry[k] = (r.x >> 16) | (r.y & 0xFFFF0000u);
                 if (g[k] != 0xFFFFFFFFu) srect[b + k * 32 + lane] = r;  // the placement reads it in order
@@ -1226,10 +1227,9 @@ cudaError_t launch_bin_sort(const igs_frame& f, int footprint, cudaStream_t st) 
 
         const uint2* rect = reinterpret_cast<const uint2*>(f.rect);
         const uint2* rg = reinterpret_cast<const uint2*>(f.ranges);
-        const DiscRef disc{rect, reinterpret_cast<const float4*>(f.disc), f.tile, 1.0f / (float)f.tile, footprint,
-                           f.tiles_x};
+        const DiscRef disc{rect, reinterpret_cast<const float4*>(f.disc), f.tile, 1.0f / (float)f.tile, footprint};
         const auto rows_count = footprint ? k_rows_count<true> : k_rows_count<false>;
-        CK(launch_pdl(rows_count, dim3(walk_blocks((const void*)rows_count, count1, cmax)), dim3(32 * kWalkWarps), count1, st, f.order, disc, rows, cmax, s.walk_h1, s.walk_rect, f.info));
+        CK(launch_pdl(rows_count, dim3(walk_blocks((const void*)rows_count, count1, cmax)), dim3(32 * kWalkWarps), count1, st, f.order, rect, disc.disc, disc.tile, disc.inv_tile, cols, rows, cmax, s.walk_h1, s.walk_rect, f.info));
         count_launches();
         CK(cudaGetLastError());
         CK(launch_pdl(k_rows_scan, dim3(rows + (s.tile_order ? 1 : 0)), dim3(kRowScanThreads), 0, st, s.walk_h1, cmax,
